@@ -101,7 +101,7 @@ def draw(rng):
                     nz=1 if two else _log(rng, 32, 128), f64=rng.random() < 0.25, m=rng.randint(2, 4),
                     passes=rng.randint(1, 2), steps=rng.randint(1, 6))
     if kind == "batch":
-        return dict(kind="batch", count=_log(rng, 16, 256), lo=64, hi=_log(rng, 128, 1024), m=rng.randint(2, 4),
+        return dict(kind="batch", count=_log(rng, 16, 256), lo=64, hi=_log(rng, 128, 1024), m=rng.choice([2, 4]),
                     sizes_seed=rng.randint(1, 10**6), steps=2 * rng.randint(1, 3))
     return dict(kind="gradient", nx=_log(rng, 96, 1200), ny=_log(rng, 96, 1200), m=rng.randint(2, 4),
                 passes=rng.randint(0, 3), sources=rng.randint(1, 96), steps=rng.randint(4, 12),
