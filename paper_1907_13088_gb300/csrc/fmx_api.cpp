@@ -653,10 +653,12 @@ fmx_status fused_step(fmx_grid *g, int nsteps, StepPre pre = nullptr) {
     const fmx::Coef<T> c0 = make_coef<T>(g->co);
     // TE/TM kernels: the TE and TM chains touch disjoint components, so the TM
     // launches go to a second stream, forked from and joined back into the
-    // grid's stream (not when profiling: the events time one stream)
+    // grid's stream (not when profiling: the events time one stream; nor on
+    // small grids, whose one launch carries both sets)
     bool two = false;
     if constexpr (sizeof(T) == 4)
-        two = nsteps > 0 && !g->prof && fmx::fused2d_pol_supported(g->geo) && c0.c6 == 1.f / 6.f;
+        two = nsteps > 0 && !g->prof && fmx::fused2d_pol_supported(g->geo) && c0.c6 == 1.f / 6.f &&
+              (g->seg_rows > 0 || fmx::fused2d_tiles(g->geo) != 1);
     if (pre && nsteps > 0) {
         fmx_status s = pre(g, 0, g->stream);
         if (s != FMX_OK) return s;

@@ -13,6 +13,11 @@
 #include "pol_tile.cuh"
 
 namespace fmx {
+
+// the step of one set (TE, TM) or of both (2) on register tiles (tile2d.cu)
+template <int SET, int M, int P, bool HJ>
+void launch_tile2d(const Geo &g, const pair2::Coef2 &c, const Fused2dArgs<float> &a, cudaStream_t s);
+
 namespace {
 
 using namespace pair2;
@@ -80,6 +85,7 @@ struct PolLauncher {
         return sh;
     }
     static void run(const Geo &g, const Coef2 &c, const Fused2dArgs<float> &a, cudaStream_t s) {
+        if (t_rows == 0 && fused2d_tiles(g)) return launch_tile2d<POL, M, P, HJ>(g, c, a, s);
         const Fused2dShape sh = shape(g);
         if (g.nx % 2 == 0 && t_l1pf)
             k_pol2d<POL, M, P, HJ, NT, true><<<sh.strips * sh.segments, NT, smem_bytes(), s>>>(a, g, c, sh.width, sh.rows,
@@ -102,6 +108,10 @@ int run_both(const Geo &g, const Coef2 &c, const Fused2dArgs<float> &a, cudaStre
     if (sh) {
         *sh = PolLauncher<TE, M, P, HJ>::shape(g);
         return 0;
+    }
+    if (!t_ev && !t_tm && t_rows == 0 && fused2d_tiles(g) == 1) {
+        launch_tile2d<2, M, P, HJ>(g, c, a, s);
+        return 1;
     }
     if (t_ev) cudaEventRecord(t_ev[0], s);
     PolLauncher<TE, M, P, HJ>::run(g, c, a, s);
