@@ -120,8 +120,7 @@ int launch_march3d_sweep(const Geo &g, const Coef<T> &c, const T *const dEp[3], 
 template <typename T>
 int launch_march3d_sweeps2(const Geo &g, const Coef<T> &c, const T *const dEp[3], const T *const in[3],
                            T *const out[3], cudaStream_t s, bool update);
-// Faraday of the 3D FP32 column-pair path; returns 0 (nothing launched) where
-// that path does not apply
+// Faraday of the 3D z-marching path
 template <typename T>
 int launch_march3d_faraday(const Geo &g, const Coef<T> &c, const T *const E[3], T *const B[3], cudaStream_t s);
 

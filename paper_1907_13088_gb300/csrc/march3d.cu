@@ -1,54 +1,54 @@
-// 3D z-marching kernels for the source (with the one-pass current filter) and
-// the sweeps of Algorithm 1.  A CTA owns a TX x TY column tile and walks a
-// segment of z planes; each input plane of the tile, with a one-cell halo in
-// x and y, is copied once into a shared-memory ring, so that every stencil of
-// the step (the A operator of Eqs. matrixA_1st..matrixA_last, the averaged
-// curl of Eqs. ampere_aux_x..z, the 27-point binomial) reads its neighbours
-// from shared memory.  The planes travel by cp.async, several planes ahead
-// of the one being computed, so no register holds data in flight: planes
-// k-1..k+1 are read while planes k+2..k+RS-2 are on their way (RS ring
-// slots), and the sweep's dE' of the thread's own cell rides in a second ring
-// of the same depth.  One __syncthreads per plane; the slot refilled after it
-// was last read in the previous plane's iteration.  The stencil arithmetic of
-// these one-column kernels (FP64, odd n_x) is the staged engine's
-// (stencil.cuh), read through a ring accessor.  The FP32 column-pair kernels
-// further down factor the A operator and the averaged curl into in-plane
-// stencils and 3-point combinations along z, so that they read one plane per
-// iteration and carry the z-combinations in registers.
+// 3D z-marching kernels for the source (with the one-pass current filter), the
+// sweeps of Algorithm 1 and the Faraday update.  A CTA owns a column tile and
+// walks a segment of z planes; each input plane of the tile, with a one-cell
+// halo in x and y, is copied once into a shared-memory ring by cp.async,
+// planes ahead of the one being computed, so that no register holds data in
+// flight; one __syncthreads per plane.  The A operator (Eqs.
+// matrixA_1st..matrixA_last) and the averaged curl (Eqs. ampere_aux_x..z) are
+// factored into in-plane stencils and 3-point combinations along z, so that an
+// iteration reads one plane and carries the z-combinations in registers.  FP32
+// grids with even n_x work on column pairs (one row per thread); FP64 grids and
+// odd n_x on single columns, four rows per thread.
 #include <cuda_runtime.h>
 
 #include <type_traits>
 
 #include "fmx_internal.h"
 #include "pair2.cuh"
-#include "stencil.cuh"
 
 namespace fmx {
 namespace {
 
-constexpr int TX = 32, TY = 8, NTH = TX * TY;  // tile and threads
-constexpr int RW = TX + 2, RH = TY + 2, PL = RW * RH;  // a tile plane with its halo
-constexpr int ZSEG = 32;                                // planes per CTA
+constexpr int TY = 8, NTH = 32 * TY, RH = TY + 2;  // pair kernels: rows of the tile, threads, rows with halo
 
-// ring slots: 8 for FP32 (five planes in flight), 4 for FP64 (one)
-template <typename T>
-struct RingDepth {
-    static constexpr int RS = sizeof(T) == 4 ? 8 : 4;
-    static constexpr int LA = RS - 3;  // copy groups in flight ahead of the plane computed
-};
-
-// component c of the ring at a shift (dx, dy in [-1, 1], dz in [-1, 1]) of
-// the thread's cell in plane k
-template <typename T>
-struct Ring {
-    const T *base;        // this component's slot-0 plane; slots are `stride` floats apart
-    int sm1, s0, sp1;     // slot offsets of planes k-1, k, k+1
-    int cell;             // (ty + 1) * RW + tx + 1
-    __device__ __forceinline__ T operator()(Pos, int dx, int dy, int dz) const {
-        const int so = dz < 0 ? sm1 : (dz > 0 ? sp1 : s0);
-        return base[so + cell + dy * RW + dx];
+// planes a segment marches over.  The CTAs on one SM share its arithmetic, so a
+// launch takes about the CTAs of the fullest SM times the planes each marches
+// (two more than it writes), and c of them resident at a time leave their
+// latencies open, which a factor 1 + 1/(2c) stands for; the segment height
+// with the least product, 4 to 64 planes, is taken (128 x 128 x 96 FP64 sweep: 24
+// planes, one CTA on each of 128 SMs, 270 us; 7 planes, 448 CTAs, 250 us).
+// tiles: CTAs per segment; res: CTAs an SM holds.
+int zseg_for(int nz, long long tiles, int res) {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
+    }();
+    int best = 1;
+    double least = 1e300;
+    for (int nseg = (nz + 63) / 64; nseg <= nz; ++nseg) {
+        const int z = (nz + nseg - 1) / nseg;
+        if (z < 4 && nseg > 1) break;
+        const long long n = (tiles * ((nz + z - 1) / z) + sms - 1) / sms;  // CTAs of the fullest SM
+        // rounds of res resident CTAs, then the rest
+        const double load = (double)(n / res) * (res + 0.5) + (n % res ? (double)(n % res) + 0.5 : 0.0);
+        if (load * (z + 2) < least) {
+            least = load * (z + 2);
+            best = z;
+        }
     }
-};
+    return best;
+}
 
 __device__ __forceinline__ int wrapm(int v, int n) { return ((v % n) + n) % n; }
 
@@ -71,178 +71,307 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// Copies of the tile's planes with their halo: a thread owns cells q = tid and
-// q = tid + NTH (when < PL) of every plane; their in-plane offsets are fixed,
-// so they are computed once.  issue(k) starts the copy of plane k (periodic)
-// of the N components into ring slot k mod RS.
+// ---------------------------------------------------------------------------
+// One column per thread (FP64, odd n_x): a tile of 32 columns x 16 rows, 128
+// threads, four rows of a column each.  FP64 arithmetic runs at 1/64 of the
+// FP32 rate on this part and bounds these kernels, so they are written for the
+// fewest operations: the factored form (see plane_terms below), differences
+// formed once and shared along the four rows of a thread, partial outputs
+// carried as FMA accumulators.  A sweep takes 54 FP64 operations per cell
+// against 135 for the 27-point stencils evaluated cell by cell, the filtered
+// source 52 against about 150.  128 x 128 x 96 FP64: sweep 685 -> 242 us, source
+// 627 -> 231 us (their operations take 213 and 189 us at the FMA rate that
+// fmx_fma_peak measures); 201 x 150 x 99 FP32: sweep 53 -> 33 us, source 68 -> 38 us.
+constexpr int CX = 32, CR = 4, CW = 4, CROWS = CR * CW, CNT = 32 * CW;
+constexpr int CPW = CX + 2, CPL = CPW * (CROWS + 2);  // row and plane of the tile with its halo
+constexpr int CCP = (CPL + CNT - 1) / CNT;             // copies of a component plane per thread
+
+// the copies of the tile's planes: plane z0 - 1 + i into ring slot i mod RS
 template <typename T, int N, int RS>
-struct AsyncPlanes {
-    const T *src[N];
-    int off0, off1;  // in-plane offsets of the thread's cells (off1 < 0: none)
-    int q0, q1;
-    __device__ __forceinline__ void init(const T *const s[N], const Geo &g, int x0, int y0) {
+struct ColPlanes {
+    int off[CCP];  // in-plane offsets of the thread's elements
+    int64_t base;  // element offset of the plane copied next, wrapped into [0, n_z)
+    int slot;
+    __device__ __forceinline__ void init(const Geo &g, int x0, int y0, int k0) {
 #pragma unroll
-        for (int c = 0; c < N; ++c) src[c] = s[c];
-        const int tid = threadIdx.y * TX + threadIdx.x;
-        q0 = tid;
-        q1 = tid + NTH < PL ? tid + NTH : -1;
-        auto off = [&](int q) {
-            const int x = wrapm(x0 - 1 + q % RW, g.nx), y = wrapm(y0 - 1 + q / RW, g.ny);
-            return y * (int)g.pitch + x;
-        };
-        off0 = off(q0);
-        off1 = q1 >= 0 ? off(q1) : -1;
-    }
-    __device__ __forceinline__ void issue(T *ring, const Geo &g, int k) const {
-        const int64_t base = (int64_t)wrapm(k, g.nz) * g.plane;
-        const int slot = k & (RS - 1);
-#pragma unroll
-        for (int c = 0; c < N; ++c) {
-            cp_async_el(ring + (slot * N + c) * PL + q0, src[c] + base + off0);
-            if (q1 >= 0) cp_async_el(ring + (slot * N + c) * PL + q1, src[c] + base + off1);
+        for (int q = 0; q < CCP; ++q) {
+            const int e = threadIdx.x + q * CNT;
+            off[q] = e < CPL ? wrapm(y0 - 1 + e / CPW, g.ny) * (int)g.pitch + wrapm(x0 - 1 + e % CPW, g.nx) : -1;
         }
+        base = (int64_t)wrapm(k0, g.nz) * g.plane;
+        slot = 0;
+    }
+    __device__ __forceinline__ void issue_next(T *ring, const T *const src[N], const Geo &g) {
+        T *dst = ring + slot * N * CPL + threadIdx.x;
+#pragma unroll
+        for (int q = 0; q < CCP; ++q) {
+            if (off[q] < 0) continue;
+#pragma unroll
+            for (int n = 0; n < N; ++n) cp_async_el(dst + n * CPL + q * CNT, src[n] + base + off[q]);
+        }
+        base += g.plane;
+        if (base == (int64_t)g.nz * g.plane) base = 0;
+        slot = slot + 1 == RS ? 0 : slot + 1;
     }
 };
 
-template <typename T, int N, int RS>
-__device__ __forceinline__ void ring_fields(Ring<T> f[N], const T *ring, int k) {
-    const int cell = (threadIdx.y + 1) * RW + threadIdx.x + 1;
-#pragma unroll
-    for (int c = 0; c < N; ++c) {
-        f[c].base = ring + c * PL;
-        f[c].sm1 = ((k - 1) & (RS - 1)) * N * PL;
-        f[c].s0 = (k & (RS - 1)) * N * PL;
-        f[c].sp1 = ((k + 1) & (RS - 1)) * N * PL;
-        f[c].cell = cell;
-    }
-}
-
-// out = dEp + A in (one sweep of Algorithm 1), 3D.  (A register window of the
-// 3 x 3 x 3 neighbourhood per component, read once per plane, was measured
-// slower: 111 registers leave 2 CTAs per SM.)
 template <typename T>
-__global__ void __launch_bounds__(NTH) k3_sweep(Geo g, Coef<T> c, const T *p0, const T *p1, const T *p2,
-                                                const T *i0, const T *i1, const T *i2, T *o0, T *o1, T *o2) {
-    constexpr int RS = RingDepth<T>::RS, LA = RingDepth<T>::LA;
+__device__ __forceinline__ T d2s(T a, T v, T b) { return (a + b) - T(2) * v; }  // a - 2 v + b
+
+// out = dEp + A in, or with UPD E = E + dEp + A in (E in place)
+constexpr int SWEEP1_RS = 4;
+template <typename T, bool UPD>
+__global__ void __launch_bounds__(CNT, sizeof(T) == 8 ? 3 : (UPD ? 4 : 6)) k3_sweep1(Geo g, Coef<T> c, const T *p0, const T *p1, const T *p2, const T *i0,
+                                                 const T *i1, const T *i2, T *o0, T *o1, T *o2, int zseg) {
+    constexpr int RS = SWEEP1_RS;
     extern __shared__ __align__(16) unsigned char m3raw[];
-    T *ring = reinterpret_cast<T *>(m3raw);  // [RS][3][PL] input planes with halo
-    T *own = ring + RS * 3 * PL;             // [RS][3][NTH] dE' of each thread's cell
+    T *ring = reinterpret_cast<T *>(m3raw);  // [RS][3][CPL]
     const T *in[3] = {i0, i1, i2};
     const T *dp[3] = {p0, p1, p2};
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int z0 = blockIdx.z * ZSEG, z1 = min(z0 + ZSEG, g.nz);
-    const int tid = threadIdx.y * TX + threadIdx.x;
-    AsyncPlanes<T, 3, RS> ld;
-    ld.init(in, g, x0, y0);
-    Pos p;
-    p.i = x0 + threadIdx.x;
-    p.j = y0 + threadIdx.y;
-    const bool inside = p.i < g.nx && p.j < g.ny;
-    const int64_t cell = (int64_t)p.j * g.pitch + p.i;
-    // copy group m: input plane z0+1+m and dE' plane z0+m (group 0 also planes
-    // z0-1 and z0); planes past the segment are not copied (empty groups keep
-    // the count)
-    auto issue = [&](int m) {
-        if (m == 0) {
-            ld.issue(ring, g, z0 - 1);
-            ld.issue(ring, g, z0);
-        }
-        if (z0 + 1 + m <= z1) ld.issue(ring, g, z0 + 1 + m);
-        const int kd = z0 + m;
-        if (inside && kd < z1) {
-            const int slot = kd & (RS - 1);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) cp_async_el(own + (slot * 3 + q) * NTH + tid, dp[q] + (int64_t)kd * g.plane + cell);
-        }
+    T *out[3] = {o0, o1, o2};
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    const int x0 = blockIdx.x * CX, y0 = blockIdx.y * CROWS;
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
+    const int np = z1 - z0 + 2;  // input planes z0-1 .. z1
+    ColPlanes<T, 3, RS> cp;
+    cp.init(g, x0, y0, z0 - 1);
+    auto issue = [&](int i) {
+        if (i < np) cp.issue_next(ring, in, g);
         cp_async_commit();
     };
 #pragma unroll
-    for (int m = 0; m < LA; ++m) issue(m);
-    for (int k = z0; k < z1; ++k) {
-        cp_async_wait<LA - 1>();  // this thread's copies of group k - z0
-        __syncthreads();          // everyone's, and every read of the slots refilled next is done
-        issue(k - z0 + LA);
-        if (inside) {
-            p.k = k;
-            Ring<T> f[3];
-            ring_fields<T, 3, RS>(f, ring, k);
-            const T *d = own + (k & (RS - 1)) * 3 * NTH + tid;
-            const int64_t idx = (int64_t)k * g.plane + cell;
-            o0[idx] = d[0] + apply_a<T, 3, 0>(f, p, c);
-            o1[idx] = d[NTH] + apply_a<T, 3, 1>(f, p, c);
-            o2[idx] = d[2 * NTH] + apply_a<T, 3, 2>(f, p, c);
+    for (int i = 0; i < RS - 1; ++i) issue(i);
+    const int x = x0 + lane, y = y0 + wy * CR;
+    const int rows = x < g.nx ? min(CR, g.ny - y) : 0;  // rows of the thread inside the grid
+    int64_t cell = (int64_t)z0 * g.plane + (int64_t)y * g.pitch + x;
+    const T bxy6 = c.bxy * c.c6, ax2 = c.ax - T(2) * c.axy;
+    T xa[CR], xb[CR], ya[CR], yb[CR], za[CR];  // partial outputs o, o+1
+#pragma unroll
+    for (int r = 0; r < CR; ++r) xa[r] = xb[r] = ya[r] = yb[r] = za[r] = T(0);
+    int slot = 0;
+    for (int i = 0; i < np; ++i) {
+        cp_async_wait<RS - 2>();
+        __syncthreads();
+        issue(i + RS - 1);
+        const T *pl = ring + slot * 3 * CPL + (wy * CR + 1) * CPW + lane + 1;
+        slot = slot + 1 == RS ? 0 : slot + 1;
+        if (rows <= 0) continue;
+        // dE' (and E^n) of the output plane this iteration completes
+        T pd[3][CR], pe[UPD ? 3 : 1][CR];
+#pragma unroll
+        for (int r = 0; r < CR; ++r)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const bool ok = i >= 2 && r < rows;
+                pd[q][r] = ok ? __ldg(dp[q] + cell + (int64_t)r * g.pitch) : T(0);
+                if (UPD) pe[UPD ? q : 0][r] = ok ? out[q][cell + (int64_t)r * g.pitch] : T(0);
+            }
+        auto V = [&](int q, int dx, int r) -> T { return pl[q * CPL + r * CPW + dx]; };
+        // what row r takes over from row r - 1
+        T ex_m = V(0, 0, -1), ex_0 = V(0, 0, 0), b_m = ex_m - V(0, -1, -1), b_0 = ex_0 - V(0, -1, 0);
+        T a_m, yp_m;
+        {
+            const T ey = V(1, 0, -1), eyr = V(1, 1, -1);
+            a_m = eyr - ey;
+            yp_m = ey + c.c6 * d2s(V(1, -1, -1), ey, eyr);
         }
+        T ez_m = V(2, 0, -1), ez_0 = V(2, 0, 0), c_m, c_0, d_m, d_0, zx_0;
+        {
+            const T er = V(2, 1, -1), er0 = V(2, 1, 0);
+            c_m = er - ez_m;
+            c_0 = er0 - ez_0;
+            d_m = d2s(V(2, -1, -1), ez_m, er);
+            d_0 = d2s(V(2, -1, 0), ez_0, er0);
+            zx_0 = ez_0 + c.c6 * d_0;
+        }
+#pragma unroll
+        for (int r = 0; r < CR; ++r) {
+            // Ex: P = Dbar_yy Ex, X = Dbar_x (Ex + P/6), Gp = Dbar_x Dbar_y Ex
+            const T ex_p = V(0, 0, r + 1), b_p = ex_p - V(0, -1, r + 1);
+            const T P = d2s(ex_p, ex_0, ex_m), X = b_0 + c.c6 * d2s(b_p, b_0, b_m), Gp = b_p - b_0;
+            // Ey: Q = Dbar_xx Ey, Y = Dbar_y (Ey + Q/6), G = Dbar_x Dbar_y Ey
+            const T ey = V(1, 0, r), eyr = V(1, 1, r);
+            const T Q = d2s(V(1, -1, r), ey, eyr), a_0 = eyr - ey, yp_0 = ey + c.c6 * Q;
+            const T Y = yp_0 - yp_m, G = a_0 - a_m;
+            // Ez: N = Dbar_x (Ez + Dbar_yy Ez / 6), Np = Dbar_y (Ez + Dbar_xx Ez / 6), T
+            const T ez_p = V(2, 0, r + 1), er_p = V(2, 1, r + 1);
+            const T c_p = er_p - ez_p, d_p = d2s(V(2, -1, r + 1), ez_p, er_p), zx_p = ez_p + c.c6 * d_p;
+            const T N = c_0 + c.c6 * d2s(c_p, c_0, c_m), Np = zx_p - zx_0;
+            const T t = c.axy * (d_p + d_m) + (c.ay * d2s(ez_p, ez_0, ez_m) + ax2 * d_0);
+            const T zh = c.byz * Y + c.bzx * X;
+            const T x1 = bxy6 * G + (c.ayz * P + c.az * ex_0), y1 = bxy6 * Gp + (c.azx * Q + c.az * ey);
+            if (i >= 2 && r < rows) {
+                // output plane z0 + i - 2 is complete
+                const int64_t o = cell + (int64_t)r * g.pitch;
+                T v[3] = {xa[r] + x1, ya[r] + y1, za[r] + zh};
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    v[q] = pd[q][r] + v[q];
+                    if (UPD) v[q] = pe[UPD ? q : 0][r] + v[q];
+                    out[q][o] = v[q];
+                }
+            }
+            xa[r] = T(-2) * x1 + (c.bzx * N + (c.bxy * G + (c.ay * P + xb[r])));
+            xb[r] = x1 - c.bzx * N;
+            ya[r] = T(-2) * y1 + (c.byz * Np + (c.bxy * Gp + (c.ax * Q + yb[r])));
+            yb[r] = y1 - c.byz * Np;
+            za[r] = t - zh;
+            ex_m = ex_0, ex_0 = ex_p, b_m = b_0, b_0 = b_p;
+            a_m = a_0, yp_m = yp_0;
+            ez_m = ez_0, ez_0 = ez_p, c_m = c_0, c_0 = c_p, d_m = d_0, d_0 = d_p, zx_0 = zx_p;
+        }
+        if (i >= 2) cell += g.plane;
     }
     cp_async_wait<0>();
 }
 
-// dE' = C_b (alpha B) - q F j, 3D, F = one (1/4, 1/2, 1/4) pass along each
-// axis (PASSES = 1) or none (PASSES = 0); HJ: a current is bound
+// dE' = C_b (alpha B) - q F j, F = one (1/4, 1/2, 1/4) pass along each axis
+// (PASSES = 1) or none (PASSES = 0); HJ: a current is bound.  The terms of
+// curl_plane_terms below, per row.
+constexpr int SOURCE1_RS = 3;
 template <typename T, int PASSES, bool HJ>
-__global__ void __launch_bounds__(NTH) k3_source(Geo g, Coef<T> c, const T *b0, const T *b1, const T *b2,
-                                                 const T *j0, const T *j1, const T *j2, T *o0, T *o1, T *o2) {
-    constexpr int N = HJ ? 6 : 3;
-    constexpr int RS = RingDepth<T>::RS, LA = RingDepth<T>::LA;
+__global__ void __launch_bounds__(CNT) k3_source1(Geo g, Coef<T> c, const T *b0, const T *b1, const T *b2, const T *j0,
+                                                  const T *j1, const T *j2, T *o0, T *o1, T *o2, int zseg) {
+    constexpr int RS = SOURCE1_RS, N = HJ ? 6 : 3;
     extern __shared__ __align__(16) unsigned char m3raw[];
-    T *ring = reinterpret_cast<T *>(m3raw);  // [RS][N][PL]
+    T *ring = reinterpret_cast<T *>(m3raw);  // [RS][N][CPL]
     const T *src[6] = {b0, b1, b2, j0, j1, j2};
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int z0 = blockIdx.z * ZSEG, z1 = min(z0 + ZSEG, g.nz);
-    AsyncPlanes<T, N, RS> ld;
-    ld.init(src, g, x0, y0);
-    // copy group m: plane z0+1+m (group 0 also planes z0-1 and z0)
-    auto issue = [&](int m) {
-        if (m == 0) {
-            ld.issue(ring, g, z0 - 1);
-            ld.issue(ring, g, z0);
-        }
-        if (z0 + 1 + m <= z1) ld.issue(ring, g, z0 + 1 + m);
+    T *out[3] = {o0, o1, o2};
+    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    const int x0 = blockIdx.x * CX, y0 = blockIdx.y * CROWS;
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
+    const int np = z1 - z0 + 2;  // input planes z0-1 .. z1
+    ColPlanes<T, N, RS> cp;
+    cp.init(g, x0, y0, z0 - 1);
+    auto issue = [&](int i) {
+        if (i < np) cp.issue_next(ring, src, g);
         cp_async_commit();
     };
 #pragma unroll
-    for (int m = 0; m < LA; ++m) issue(m);
-    Pos p;
-    p.i = x0 + threadIdx.x;
-    p.j = y0 + threadIdx.y;
-    const bool inside = p.i < g.nx && p.j < g.ny;
-    for (int k = z0; k < z1; ++k) {
-        cp_async_wait<LA - 1>();
+    for (int i = 0; i < RS - 1; ++i) issue(i);
+    const int x = x0 + lane, y = y0 + wy * CR;
+    const int rows = x < g.nx ? min(CR, g.ny - y) : 0;
+    int64_t cell = (int64_t)z0 * g.plane + (int64_t)y * g.pitch + x;
+    const T kyc6 = c.ky * c.c6, nkxc6 = -(c.kx * c.c6);
+    // the current's factor, with PASSES = 1 over the integer weights' 64 (exact)
+    const T qj = PASSES == 1 ? c.q * T(1.0 / 64.0) : c.q;
+    T xa[CR], xb[CR], ya[CR], yb[CR], za[CR];
+    T up[CR], wp[CR];  // U and W of the plane before
+    T jz[HJ ? 3 : 1][2][CR];  // x-y binomial of planes j-2, j-1 (PASSES = 0: the current itself)
+#pragma unroll
+    for (int r = 0; r < CR; ++r) {
+        xa[r] = xb[r] = ya[r] = yb[r] = za[r] = up[r] = wp[r] = T(0);
+        if (HJ)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) jz[HJ ? q : 0][0][r] = jz[HJ ? q : 0][1][r] = T(0);
+    }
+    int slot = 0;
+    for (int i = 0; i < np; ++i) {
+        cp_async_wait<RS - 2>();
         __syncthreads();
-        issue(k - z0 + LA);
-        if (inside) {
-            p.k = k;
-            Ring<T> f[N];
-            ring_fields<T, N, RS>(f, ring, k);
-            T d[3] = {curl_alpha_b<T, 3, 0>(f, p, c), curl_alpha_b<T, 3, 1>(f, p, c), curl_alpha_b<T, 3, 2>(f, p, c)};
+        issue(i + RS - 1);
+        const T *pl = ring + slot * N * CPL + (wy * CR + 1) * CPW + lane + 1;
+        slot = slot + 1 == RS ? 0 : slot + 1;
+        if (rows <= 0) continue;
+        auto V = [&](int q, int dx, int r) -> T { return pl[q * CPL + r * CPW + dx]; };
+        auto wx = [&](int r) { return V(0, 0, r) + c.c6 * d2s(V(0, -1, r), V(0, 0, r), V(0, 1, r)); };  // alpha_x Bx
+        auto jr = [&](int q, int r) { return (V(3 + q, -1, r) + V(3 + q, 1, r)) + T(2) * V(3 + q, 0, r); };
+        T w_m = wx(-1), bz_m = V(2, 0, -1);
+        T by_m = V(1, 0, -1), by_0 = V(1, 0, 0), u_m = by_m - V(1, -1, -1), u_0 = by_0 - V(1, -1, 0);
+        T s_m[3], s_0[3];
+        if constexpr (HJ && PASSES == 1) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                s_m[q] = jr(q, -1);
+                s_0[q] = jr(q, 0);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < CR; ++r) {
+            const T by_p = V(1, 0, r + 1), u_p = by_p - V(1, -1, r + 1);
+            const T U = by_0 + c.c6 * d2s(by_p, by_0, by_m), Ux = u_0 + c.c6 * d2s(u_p, u_0, u_m);
+            const T W = wx(r), Wy = W - w_m;
+            const T bz = V(2, 0, r), Vy = bz - bz_m, Vx = bz - V(2, -1, r);
+            const T x1 = kyc6 * Vy, y1 = nkxc6 * Vx;
+            T jn[3];
             if constexpr (HJ) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    T jf;
+                for (int q = 0; q < 3; ++q) {
                     if constexpr (PASSES == 1) {
-                        // separable binomial: weights (1, 2, 1)/4 per axis
-                        jf = T(0);
-#pragma unroll
-                        for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-                            for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-                                for (int dx = -1; dx <= 1; ++dx) {
-                                    const T w = T((2 - dx * dx) * (2 - dy * dy) * (2 - dz * dz)) * T(1.0 / 64.0);
-                                    jf += w * f[3 + a](p, dx, dy, dz);
-                                }
+                        const T s_p = jr(q, r + 1);
+                        jn[q] = (s_p + s_m[q]) + T(2) * s_0[q];
+                        s_m[q] = s_0[q];
+                        s_0[q] = s_p;
                     } else {
-                        jf = f[3 + a](p, 0, 0, 0);
+                        jn[q] = V(3 + q, 0, r);
                     }
-                    d[a] -= c.q * jf;
                 }
             }
-            const int64_t idx = (int64_t)k * g.plane + (int64_t)p.j * g.pitch + p.i;
-            o0[idx] = d[0];
-            o1[idx] = d[1];
-            o2[idx] = d[2];
+            if (i >= 2 && r < rows) {
+                const int64_t o = cell + (int64_t)r * g.pitch;
+                T d[3] = {xa[r] + x1, ya[r] + y1, za[r]};
+                if constexpr (HJ) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if constexpr (PASSES == 1) d[q] -= qj * ((jz[q][0][r] + jn[q]) + T(2) * jz[q][1][r]);
+                        else d[q] -= qj * jz[q][1][r];
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 3; ++q) out[q][o] = d[q];
+            }
+            // the z-differences of U and W before their factor: on smooth fields
+            // a difference is exact where the products' sum would round at |B|
+            xa[r] = T(-2) * x1 + (c.ky * Vy + (xb[r] - c.kz * (U - up[r])));
+            xb[r] = x1;
+            ya[r] = T(-2) * y1 + (c.kz * (W - wp[r]) + (yb[r] - c.kx * Vx));
+            yb[r] = y1;
+            up[r] = U;
+            wp[r] = W;
+            za[r] = c.kx * Ux - c.ky * Wy;
+            if constexpr (HJ) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    jz[q][0][r] = jz[q][1][r];
+                    jz[q][1][r] = jn[q];
+                }
+            }
+            w_m = W, bz_m = bz;
+            by_m = by_0, by_0 = by_p, u_m = u_0, u_0 = u_p;
         }
+        if (i >= 2) cell += g.plane;
     }
     cp_async_wait<0>();
+}
+
+// B -= c dt curl E^{n+1} (Eqs. faraday_x..z), forward differences: a thread
+// walks the planes of its column, E of the plane above carried over; the
+// neighbours x+1 and y+1 come through L1.  Bound by memory; the
+// one-thread-per-cell kernel spent its time on periodic 64-bit indices (201 x
+// 150 x 99 FP32 26.5 -> 20.5 us).
+template <typename T>
+__global__ void __launch_bounds__(256) k3_faraday1(Geo g, Coef<T> c, const T *__restrict__ e0, const T *__restrict__ e1,
+                                                   const T *__restrict__ e2, T *__restrict__ b0, T *__restrict__ b1,
+                                                   T *__restrict__ b2, int zseg) {
+    const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (x >= g.nx || y >= g.ny) return;
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
+    const int o = y * (int)g.pitch + x;
+    const int ox = o + (x + 1 < g.nx ? 1 : 1 - g.nx), oy = o + (y + 1 < g.ny ? (int)g.pitch : -(g.ny - 1) * (int)g.pitch);
+    int64_t z = (int64_t)z0 * g.plane;
+    T ex = e0[z + o], ey = e1[z + o];
+    for (int k = z0; k < z1; ++k) {
+        const int64_t zn = k + 1 < g.nz ? z + g.plane : 0;
+        const T ez = e2[z + o], exn = e0[zn + o], eyn = e1[zn + o];
+        const T bx = b0[z + o], by = b1[z + o], bz = b2[z + o];
+        const T ezx = e2[z + ox], ezy = e2[z + oy], eyx = e1[z + ox], exy = e0[z + oy];
+        b0[z + o] = (bx - c.ky * (ezy - ez)) + c.kz * (eyn - ey);
+        b1[z + o] = (by - c.kz * (exn - ex)) + c.kx * (ezx - ez);
+        b2[z + o] = (bz - c.kx * (eyx - ey)) + c.ky * (exy - ex);
+        ex = exn;
+        ey = eyn;
+        z = zn;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -259,6 +388,7 @@ using pair2::f2;
 constexpr int TXP = 32, TX2 = 2 * TXP;              // threads along x, columns of the tile
 constexpr int RW2 = TX2 + 4, PL2 = RW2 * RH;         // smem row and plane (one component)
 constexpr int NPC = TXP * RH, NCP2 = NPC + 2 * RH;  // pair copies and halo copies per plane
+constexpr int FAR_RS = 8;    // ring slots of the pair Faraday update
 constexpr int SWEEP_RS = 8;  // ring slots of the pair sweep: one plane read, seven in flight
 
 struct Coef3P {
@@ -270,52 +400,6 @@ __device__ __forceinline__ f2 ck(const Coef3P &c) {
     return AX == 0 ? c.kx : (AX == 1 ? c.ky : c.kz);
 }
 
-template <int AX>
-__device__ __forceinline__ f2 cdiag(const Coef3P &c) {
-    return AX == 0 ? c.ax : (AX == 1 ? c.ay : c.az);
-}
-template <int AX>
-__device__ __forceinline__ f2 cpair(const Coef3P &c) {
-    return AX == 0 ? c.ayz : (AX == 1 ? c.azx : c.axy);
-}
-template <int THIRD>
-__device__ __forceinline__ f2 ccross(const Coef3P &c) {
-    return THIRD == 0 ? c.byz : (THIRD == 1 ? c.bzx : c.bxy);
-}
-
-// Dbar_{ax ax} of component q at offset (ox, oy, oz), on pairs
-template <int Q, int AX, typename F>
-__device__ __forceinline__ f2 d2p(const F &V, int ox, int oy, int oz) {
-    constexpr int ex = AX == 0, ey = AX == 1, ez = AX == 2;
-    return pair2::fma(V(Q, ox, oy, oz), pair2::m2(), pair2::add(V(Q, ox + ex, oy + ey, oz + ez), V(Q, ox - ex, oy - ey, oz - ez)));
-}
-
-// (A dE)_A on a column pair: the operator of apply_a (stencil.cuh) in 3D
-template <int A, typename F>
-__device__ __forceinline__ f2 apply_a2(const F &V, const Coef3P &c) {
-    using namespace pair2;
-    constexpr int B = (A + 1) % 3, C = (A + 2) % 3;
-    constexpr int bx = B == 0, by = B == 1, bz = B == 2, cx = C == 0, cy = C == 1, cz = C == 2;
-    const f2 dB = d2p<A, B>(V, 0, 0, 0);
-    f2 r = mul(cdiag<B>(c), dB);
-    r = fma(cdiag<C>(c), d2p<A, C>(V, 0, 0, 0), r);
-    const f2 dd = fma(dB, m2(), add(d2p<A, B>(V, cx, cy, cz), d2p<A, B>(V, -cx, -cy, -cz)));
-    r = fma(cpair<A>(c), dd, r);
-    // A_AB E_B with weight (1 + Dbar_CC / 6) at (o_A, o_B) = (1,0), (1,-1), (0,0), (0,-1)
-    auto wb = [&](int oa, int ob) {
-        const int ox = (A == 0) * oa + bx * ob, oy = (A == 1) * oa + by * ob, oz = (A == 2) * oa + bz * ob;
-        return fma(c.c6, d2p<B, C>(V, ox, oy, oz), V(B, ox, oy, oz));
-    };
-    r = fma(ccross<C>(c), fma(add(wb(1, -1), wb(0, 0)), m1(), add(wb(1, 0), wb(0, -1))), r);
-    // A_AC E_C with weight (1 + Dbar_BB / 6) at (o_A, o_C) = (1,0), (1,-1), (0,0), (0,-1)
-    auto wc = [&](int oa, int oc) {
-        const int ox = (A == 0) * oa + cx * oc, oy = (A == 1) * oa + cy * oc, oz = (A == 2) * oa + cz * oc;
-        return fma(c.c6, d2p<C, B>(V, ox, oy, oz), V(C, ox, oy, oz));
-    };
-    r = fma(ccross<B>(c), fma(add(wc(1, -1), wc(0, 0)), m1(), add(wc(1, 0), wc(0, -1))), r);
-    return r;
-}
-
 // a thread's (at most two) copy items of a component plane, and the plane the
 // z-march copies next: its index unwrapped (which picks the ring slot) and
 // the element offset of the plane wrapped periodically, advanced one plane
@@ -323,7 +407,7 @@ __device__ __forceinline__ f2 apply_a2(const F &V, const Coef3P &c) {
 struct PairCopies {
     int s[2], o[2];  // smem index within a component plane (-1: none), global in-plane offset
     bool w[2];       // column pair (8 bytes) or halo column (4 bytes)
-    int ku;          // next plane, unwrapped
+    int ku;          // planes copied so far
     int64_t off;     // element offset of that plane wrapped into [0, n_z)
     __device__ __forceinline__ void init(const Geo &g, int x0, int y0, int k0) {
         const int tid = threadIdx.y * TXP + threadIdx.x;
@@ -349,10 +433,10 @@ struct PairCopies {
                 o[r] = y * (int)g.pitch + x;
             }
         }
-        ku = k0;
+        ku = 0;
         off = (int64_t)wrapm(k0, g.nz) * g.plane;
     }
-    // copies plane ku of the N components into ring slot ku mod RS, then
+    // copies the next plane of the N components into ring slot ku mod RS, then
     // moves on to the next plane
     template <int RS, int N = 3>
     __device__ __forceinline__ void issue_next(float *ring, const float *const src[N], const Geo &g) {
@@ -447,7 +531,7 @@ __device__ __forceinline__ PlaneTerms plane_terms(const F &V, const Coef3P &c, f
 template <bool UPD>
 __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, const float *p0, const float *p1,
                                                              const float *p2, const float *i0, const float *i1,
-                                                             const float *i2, float *o0, float *o1, float *o2) {
+                                                             const float *i2, float *o0, float *o1, float *o2, int zseg) {
     using namespace pair2;
     constexpr int RS = SWEEP_RS;
     extern __shared__ __align__(16) unsigned char m3raw[];
@@ -456,7 +540,7 @@ __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, c
     const float *dp[3] = {p0, p1, p2};
     float *out[3] = {o0, o1, o2};
     const int x0 = blockIdx.x * TX2, y0 = blockIdx.y * TY;
-    const int z0 = blockIdx.z * ZSEG, z1 = min(z0 + ZSEG, g.nz);
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
     const int np = z1 - z0 + 2;  // input planes z0-1 .. z1
     PairCopies cp;
     cp.init(g, x0, y0, z0 - 1);
@@ -498,7 +582,7 @@ __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, c
         __syncthreads();
         issue(i + RS - 1);
         if (inside) {
-            const float *pl = ring + ((z0 - 1 + i) & (RS - 1)) * 3 * PL2 + c0;  // the copy's slot of plane z0-1+i
+            const float *pl = ring + (i & (RS - 1)) * 3 * PL2 + c0;  // the copy's slot of plane z0-1+i
             auto V = [&](int q, int dx, int dy) -> f2 {
                 const float *row = pl + q * PL2 + dy * RW2;
                 const f2 pr = *reinterpret_cast<const float2 *>(row);
@@ -582,7 +666,7 @@ __device__ __forceinline__ CurlTerms curl_plane_terms(const F &V, const Coef3P &
 template <int RS, int PASSES, bool HJ>
 __global__ void __launch_bounds__(NTH, 3) k3_source2(Geo g, Coef3P c, const float *b0, const float *b1,
                                                     const float *b2, const float *j0, const float *j1,
-                                                    const float *j2, float *o0, float *o1, float *o2) {
+                                                    const float *j2, float *o0, float *o1, float *o2, int zseg) {
     using namespace pair2;
     constexpr int N = HJ ? 6 : 3;
     extern __shared__ __align__(16) unsigned char m3raw[];
@@ -590,7 +674,7 @@ __global__ void __launch_bounds__(NTH, 3) k3_source2(Geo g, Coef3P c, const floa
     const float *src[6] = {b0, b1, b2, j0, j1, j2};
     float *out[3] = {o0, o1, o2};
     const int x0 = blockIdx.x * TX2, y0 = blockIdx.y * TY;
-    const int z0 = blockIdx.z * ZSEG, z1 = min(z0 + ZSEG, g.nz);
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
     const int np = z1 - z0 + 2;  // input planes z0-1 .. z1
     PairCopies cp;
     cp.init(g, x0, y0, z0 - 1);
@@ -617,7 +701,7 @@ __global__ void __launch_bounds__(NTH, 3) k3_source2(Geo g, Coef3P c, const floa
         __syncthreads();
         issue(i + RS - 1);
         if (inside) {
-            const float *pl = ring + ((z0 - 1 + i) & (RS - 1)) * N * PL2 + c0;  // the copy's slot of plane z0-1+i
+            const float *pl = ring + (i & (RS - 1)) * N * PL2 + c0;  // the copy's slot of plane z0-1+i
             auto V = [&](int q, int dx, int dy) -> f2 {
                 const float *row = pl + q * PL2 + dy * RW2;
                 const f2 pr = *reinterpret_cast<const float2 *>(row);
@@ -690,15 +774,15 @@ __device__ __forceinline__ f2 curl_e2(const F &V, const Coef3P &c) {
 }
 
 __global__ void __launch_bounds__(NTH, 3) k3_faraday2(Geo g, Coef3P c, const float *e0, const float *e1,
-                                                     const float *e2, float *b0, float *b1, float *b2) {
+                                                     const float *e2, float *b0, float *b1, float *b2, int zseg) {
     using namespace pair2;
-    constexpr int RS = RingDepth<float>::RS, LA = RingDepth<float>::LA;
+    constexpr int RS = FAR_RS, LA = RS - 3;  // LA: copy groups in flight ahead of the plane computed
     extern __shared__ __align__(16) unsigned char m3raw[];
     float *ring = reinterpret_cast<float *>(m3raw);  // [RS][3][PL2] E^{n+1} planes
     const float *in[3] = {e0, e1, e2};
     float *bo[3] = {b0, b1, b2};
     const int x0 = blockIdx.x * TX2, y0 = blockIdx.y * TY;
-    const int z0 = blockIdx.z * ZSEG, z1 = min(z0 + ZSEG, g.nz);
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
     PairCopies cp;
     cp.init(g, x0, y0, z0);
     const int px = x0 + 2 * threadIdx.x, py = y0 + threadIdx.y;
@@ -734,7 +818,7 @@ __global__ void __launch_bounds__(NTH, 3) k3_faraday2(Geo g, Coef3P c, const flo
         for (int q = 0; q < 3; ++q) bv[q] = pb[b][q];
         ldown(k + 2, b);
         if (inside) {
-            const int s0 = (k & (RS - 1)) * 3 * PL2, sp1 = ((k + 1) & (RS - 1)) * 3 * PL2;
+            const int s0 = ((k - z0) & (RS - 1)) * 3 * PL2, sp1 = ((k - z0 + 1) & (RS - 1)) * 3 * PL2;
             auto V = [&](int q, int dx, int dy, int dz) -> f2 {
                 const float *row = ring + (dz > 0 ? sp1 : s0) + q * PL2 + c0 + dy * RW2;
                 const f2 pr = *reinterpret_cast<const float2 *>(row);
@@ -778,7 +862,7 @@ constexpr int FNI = (FRW / 2) * FIR;   // pair copies per input plane and compon
 template <bool UPD>
 __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const float *p0, const float *p1,
                                                      const float *p2, const float *i0, const float *i1,
-                                                     const float *i2, float *o0, float *o1, float *o2) {
+                                                     const float *i2, float *o0, float *o1, float *o2, int zseg) {
     using namespace pair2;
     extern __shared__ __align__(16) unsigned char m3raw[];
     float *ring = reinterpret_cast<float *>(m3raw);  // [FRS][3][FIPL] input planes, halo 2
@@ -787,7 +871,7 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
     const float *dp[3] = {p0, p1, p2};
     float *out[3] = {o0, o1, o2};
     const int x0 = blockIdx.x * TX2, y0 = blockIdx.y * TY;
-    const int z0 = blockIdx.z * ZSEG, z1 = min(z0 + ZSEG, g.nz);
+    const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
     const int nin = z1 - z0 + 4;  // input planes z0-2 .. z1+1
     const int tid = threadIdx.x;
     const int64_t vol = (int64_t)g.nz * g.plane;
@@ -809,7 +893,7 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
     // copy group i: input plane z0-2+i (empty past the last)
     auto issue = [&](int i) {
         if (i < nin) {
-            float *slot = ring + ((z0 - 2 + i) & (FRS - 1)) * 3 * FIPL;
+            float *slot = ring + (i & (FRS - 1)) * 3 * FIPL;
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
                 if (cs[r] < 0) continue;
@@ -862,7 +946,7 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
         // A stage: input plane z0-2+i; completes first-sweep plane z0+i-3 (i >= 2)
         if (hasA && i < nin) {
             if (i == 1) load_a();  // dE' of plane z0-1
-            const float *pl = ring + ((z0 - 2 + i) & (FRS - 1)) * 3 * FIPL + cA;
+            const float *pl = ring + (i & (FRS - 1)) * 3 * FIPL + cA;
             auto V = [&](int q, int dx, int dy) -> f2 {
                 const float *row = pl + q * FIPL + dy * FRW;
                 const f2 pr = *reinterpret_cast<const float2 *>(row);
@@ -870,7 +954,7 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
             };
             const PlaneTerms t = plane_terms(V, c, bxy6);
             if (i >= 2) {
-                float *dst = abuf + ((z0 + i - 3) & 1) * 3 * FAPL + wA;
+                float *dst = abuf + ((i + 1) & 1) * 3 * FAPL + wA;
                 *reinterpret_cast<float2 *>(dst) = add(pa_d[0], add(ax_a, t.x1));
                 *reinterpret_cast<float2 *>(dst + FAPL) = add(pa_d[1], add(ay_a, t.y1));
                 *reinterpret_cast<float2 *>(dst + 2 * FAPL) = add(pa_d[2], add(az_a, t.zh));
@@ -885,7 +969,7 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
         // B stage: first-sweep plane z0+i-4 (i >= 3); completes output plane z0+i-5 (i >= 5)
         if (hasB && i >= 3) {
             if (i == 4) load_b(outB, bcell);  // output z0
-            const float *pl = abuf + ((z0 + i - 4) & 1) * 3 * FAPL + cB;
+            const float *pl = abuf + (i & 1) * 3 * FAPL + cB;
             auto V = [&](int q, int dx, int dy) -> f2 {
                 const float *row = pl + q * FAPL + dy * FRW;
                 const f2 pr = *reinterpret_cast<const float2 *>(row);
@@ -915,32 +999,44 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
     cp_async_wait<0>();
 }
 
-inline dim3 grid3(const Geo &g) { return dim3((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + ZSEG - 1) / ZSEG); }
+// launch grid of a kernel with CTAs of tx columns x ty rows, zseg planes each
+dim3 grid_of(const Geo &g, int tx, int ty, int res, int *zseg) {
+    const dim3 t((g.nx + tx - 1) / tx, (g.ny + ty - 1) / ty);
+    *zseg = zseg_for(g.nz, (long long)t.x * t.y, res);
+    return dim3(t.x, t.y, (g.nz + *zseg - 1) / *zseg);
+}
+// allows the dynamic shared memory and returns the CTAs an SM holds
+template <typename K>
+int resident(K k, int threads, size_t bytes) {
+    int n = 0;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, bytes) == cudaSuccess && n > 0 ? n : 1;
+}
 
 }  // namespace
 
 bool march3d_supported(int dims, int passes) { return dims == 3 && passes >= 0 && passes <= 1; }
 
-template <typename T, int N>
-size_t ring_bytes() {
-    return (size_t)RingDepth<T>::RS * N * PL * sizeof(T);
-}
-template <typename T>
-size_t sweep_bytes() {
-    return ring_bytes<T, 3>() + (size_t)RingDepth<T>::RS * 3 * NTH * sizeof(T);
-}
-
 template <typename T, int PASSES, bool HJ>
 void run_source(const Geo &g, const Coef<T> &c, const T *const B[3], const T *const J[3], T *const out[3],
                 cudaStream_t s) {
-    constexpr int N = HJ ? 6 : 3;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k3_source<T, PASSES, HJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes<T, N>());
-        attr = true;
-    }
-    k3_source<T, PASSES, HJ><<<grid3(g), dim3(TX, TY), ring_bytes<T, N>(), s>>>(
-        g, c, B[0], B[1], B[2], HJ ? J[0] : nullptr, HJ ? J[1] : nullptr, HJ ? J[2] : nullptr, out[0], out[1], out[2]);
+    constexpr size_t bytes = (size_t)SOURCE1_RS * (HJ ? 6 : 3) * CPL * sizeof(T);
+    static const int res = resident(k3_source1<T, PASSES, HJ>, CNT, bytes);
+    int zseg;
+    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg);
+    k3_source1<T, PASSES, HJ><<<grid, CNT, bytes, s>>>(g, c, B[0], B[1], B[2], HJ ? J[0] : nullptr, HJ ? J[1] : nullptr,
+                                                       HJ ? J[2] : nullptr, out[0], out[1], out[2], zseg);
+}
+
+template <typename T, bool UPD>
+void run_sweep1(const Geo &g, const Coef<T> &c, const T *const dEp[3], const T *const in[3], T *const out[3],
+                cudaStream_t s) {
+    constexpr size_t bytes = (size_t)SWEEP1_RS * 3 * CPL * sizeof(T);
+    static const int res = resident(k3_sweep1<T, UPD>, CNT, bytes);
+    int zseg;
+    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg);
+    k3_sweep1<T, UPD><<<grid, CNT, bytes, s>>>(g, c, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0], out[1],
+                                               out[2], zseg);
 }
 
 bool pair_path(const Geo &g, float *) { return g.nx % 2 == 0 && g.pitch % 2 == 0; }
@@ -958,15 +1054,12 @@ void run_source2(const Geo &g, const Coef<float> &c, const float *const B[3], co
                  float *const out[3], cudaStream_t s) {
     constexpr int N = HJ ? 6 : 3;
     constexpr size_t bytes = (size_t)SRC_RS * N * PL2 * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k3_source2<SRC_RS, PASSES, HJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        attr = true;
-    }
-    const dim3 grid((g.nx + TX2 - 1) / TX2, (g.ny + TY - 1) / TY, (g.nz + ZSEG - 1) / ZSEG);
+    static const int res = resident(k3_source2<SRC_RS, PASSES, HJ>, NTH, bytes);
+    int zseg;
+    const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
     k3_source2<SRC_RS, PASSES, HJ><<<grid, dim3(TXP, TY), bytes, s>>>(
         g, coef3p(c), B[0], B[1], B[2], HJ ? J[0] : nullptr, HJ ? J[1] : nullptr, HJ ? J[2] : nullptr, out[0], out[1],
-        out[2]);
+        out[2], zseg);
 }
 bool pair_path(const Geo &, double *) { return false; }
 
@@ -974,29 +1067,23 @@ template <bool UPD>
 void run_sweep2(const Geo &g, const Coef<float> &c, const float *const dEp[3], const float *const in[3],
                 float *const out[3], cudaStream_t s) {
     constexpr size_t bytes = (size_t)SWEEP_RS * 3 * PL2 * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k3_sweep2<UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        attr = true;
-    }
+    static const int res = resident(k3_sweep2<UPD>, NTH, bytes);
     const Coef3P cp = coef3p(c);
-    const dim3 grid((g.nx + TX2 - 1) / TX2, (g.ny + TY - 1) / TY, (g.nz + ZSEG - 1) / ZSEG);
+    int zseg;
+    const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
     k3_sweep2<UPD><<<grid, dim3(TXP, TY), bytes, s>>>(g, cp, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0],
-                                                     out[1], out[2]);
+                                                     out[1], out[2], zseg);
 }
 
 template <bool UPD>
 void run_sweeps2f(const Geo &g, const Coef<float> &c, const float *const dEp[3], const float *const in[3],
                   float *const out[3], cudaStream_t s) {
     constexpr size_t bytes = ((size_t)FRS * 3 * FIPL + (size_t)2 * 3 * FAPL) * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k3_sweeps2f<UPD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        attr = true;
-    }
-    const dim3 grid((g.nx + TX2 - 1) / TX2, (g.ny + TY - 1) / TY, (g.nz + ZSEG - 1) / ZSEG);
+    static const int res = resident(k3_sweeps2f<UPD>, FNT, bytes);
+    int zseg;
+    const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
     k3_sweeps2f<UPD><<<grid, FNT, bytes, s>>>(g, coef3p(c), dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0],
-                                             out[1], out[2]);
+                                             out[1], out[2], zseg);
 }
 
 template <typename T>
@@ -1033,18 +1120,18 @@ template <typename T>
 int launch_march3d_faraday(const Geo &g, const Coef<T> &c, const T *const E[3], T *const B[3], cudaStream_t s) {
     if constexpr (std::is_same<T, float>::value) {
         if (pair_path(g, (float *)nullptr)) {
-            constexpr size_t bytes = (size_t)RingDepth<float>::RS * 3 * PL2 * sizeof(float);
-            static bool attr = false;
-            if (!attr) {
-                cudaFuncSetAttribute(k3_faraday2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-                attr = true;
-            }
-            const dim3 grid((g.nx + TX2 - 1) / TX2, (g.ny + TY - 1) / TY, (g.nz + ZSEG - 1) / ZSEG);
-            k3_faraday2<<<grid, dim3(TXP, TY), bytes, s>>>(g, coef3p(c), E[0], E[1], E[2], B[0], B[1], B[2]);
+            constexpr size_t bytes = (size_t)FAR_RS * 3 * PL2 * sizeof(float);
+            static const int res = resident(k3_faraday2, NTH, bytes);
+            int zseg;
+    const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
+            k3_faraday2<<<grid, dim3(TXP, TY), bytes, s>>>(g, coef3p(c), E[0], E[1], E[2], B[0], B[1], B[2], zseg);
             return 1;
         }
     }
-    return 0;  // FP64 or odd n_x: the caller launches the one-thread-per-cell kernel
+    int zseg;
+    const dim3 grid = grid_of(g, 32, 8, 8, &zseg);
+    k3_faraday1<T><<<grid, 256, 0, s>>>(g, c, E[0], E[1], E[2], B[0], B[1], B[2], zseg);
+    return 1;
 }
 
 template <typename T>
@@ -1057,14 +1144,8 @@ int launch_march3d_sweep(const Geo &g, const Coef<T> &c, const T *const dEp[3], 
             return 1;
         }
     }
-    if (update) return 0;  // the scalar sweep does not fuse the update: the caller launches it
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k3_sweep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_bytes<T>());
-        attr = true;
-    }
-    k3_sweep<T><<<grid3(g), dim3(TX, TY), sweep_bytes<T>(), s>>>(g, c, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2],
-                                                                   out[0], out[1], out[2]);
+    if (update) run_sweep1<T, true>(g, c, dEp, in, out, s);
+    else run_sweep1<T, false>(g, c, dEp, in, out, s);
     return 1;
 }
 
