@@ -408,6 +408,28 @@ fmx_status filter_in_place(fmx_grid *g, T *f, int passes) {
     return check_launch(g, "filter kernel launch");
 }
 
+// The same on several components (at most 6) at once.  The scratch is what no
+// state lives in between steps: the fused engine's other state set, the staged
+// layout's dEa and dEb elsewhere.
+template <typename T>
+fmx_status filter_fields(fmx_grid *g, T *const f[], int n, int passes) {
+    T *scratch[6];
+    for (int q = 0; q < 6; ++q) {
+        if (g->engine == FMX_ENGINE_FUSED) scratch[q] = (T *)(q < 3 ? g->buf.E[1 - g->cur][q] : g->buf.B[1 - g->cur][q - 3]);
+        else scratch[q] = (T *)(q < 3 ? g->dEa[q] : g->dEb[q - 3]);
+    }
+    const int nl = passes > 0 ? fmx::launch_filter_fields<T>(g->geo, g->p.dims, passes, n, f, scratch, g->stream) : 0;
+    if (nl) {
+        g->launches += nl;
+        return check_launch(g, "filter kernel launch");
+    }
+    for (int q = 0; q < n; ++q) {
+        fmx_status s = filter_in_place<T>(g, f[q], passes);
+        if (s != FMX_OK) return s;
+    }
+    return FMX_OK;
+}
+
 // Filters the current into the jf workspace (out of place; J is unchanged)
 // and returns in jsrc the arrays the source stage should read.
 template <typename T>
@@ -559,10 +581,8 @@ fmx_status staged_step(fmx_grid *g) {
     s = check_launch(g, "staged step launch");
     if (s != FMX_OK) return s;
     if (g->p.filter_target == FMX_FILTER_FIELDS && g->p.filter_passes > 0) {
-        for (int q = 0; q < 3; ++q) {
-            if ((s = filter_in_place<T>(g, P.E[q], g->p.filter_passes)) != FMX_OK) return s;
-            if ((s = filter_in_place<T>(g, P.B[q], g->p.filter_passes)) != FMX_OK) return s;
-        }
+        T *const f[6] = {P.E[0], P.E[1], P.E[2], P.B[0], P.B[1], P.B[2]};
+        if ((s = filter_fields<T>(g, f, 6, g->p.filter_passes)) != FMX_OK) return s;
     }
     return FMX_OK;
 }
@@ -1052,11 +1072,21 @@ fmx_status fmx_filter(fmx_grid *g, unsigned mask, int passes) {
     if (mask & ~(unsigned)(FMX_E | FMX_B | FMX_J)) return fail(FMX_EINVAL, "bad mask");
     if ((mask & FMX_J) && !g->buf.J[0]) return fail(FMX_ESTATE, "no J buffers bound");
     if (mask && passes > 0 && !cellwise_launch_ok(&g->p)) return cellwise_limit_fail("fmx_filter");
-    for (int c = 0; c < 9; ++c) {
-        if (!(mask & (1u << c))) continue;
-        void *f = c < 3 ? g->buf.E[g->cur][c] : (c < 6 ? g->buf.B[g->cur][c - 3] : g->buf.J[c - 6]);
-        fmx_status s = g->p.precision == FMX_F64 ? filter_in_place<double>(g, (double *)f, passes)
-                                                 : filter_in_place<float>(g, (float *)f, passes);
+    // the components of the state, then those of the current
+    for (int first : {0, 6}) {
+        void *f[6];
+        int n = 0;
+        for (int c = first; c < (first ? 9 : 6); ++c)
+            if (mask & (1u << c)) f[n++] = c < 3 ? g->buf.E[g->cur][c] : (c < 6 ? g->buf.B[g->cur][c - 3] : g->buf.J[c - 6]);
+        if (n == 0) continue;
+        double *fd[6];
+        float *ff[6];
+        for (int q = 0; q < n; ++q) {
+            fd[q] = (double *)f[q];
+            ff[q] = (float *)f[q];
+        }
+        fmx_status s = g->p.precision == FMX_F64 ? filter_fields<double>(g, fd, n, passes)
+                                                 : filter_fields<float>(g, ff, n, passes);
         if (s != FMX_OK) return s;
     }
     return FMX_OK;

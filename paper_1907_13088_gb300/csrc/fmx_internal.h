@@ -73,6 +73,13 @@ int64_t staged_partial_slots(const Geo &g);
 template <typename T>
 int launch_filter_pass(const Geo &g, int dims, const T *in, T *out, int axis, cudaStream_t s);
 
+// `passes` binomial passes along every active axis of n (at most 6) components,
+// in place through as many scratch arrays, in two launches.  Returns 0 (nothing
+// launched) where the kernels are not instantiated (passes above 3, or a grid
+// beyond the flattened launch limits).
+template <typename T>
+int launch_filter_fields(const Geo &g, int dims, int passes, int n, T *const f[], T *const scratch[], cudaStream_t s);
+
 template <typename T>
 int launch_staged_source(const Geo &g, int dims, const Coef<T> &c, const StagedPtrs<T> &p,
                          const T *const jsrc[3], cudaStream_t s, bool norm);
