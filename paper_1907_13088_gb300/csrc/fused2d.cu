@@ -19,6 +19,14 @@
 // read from HBM and only E^{n+1}, B^{n+3/2} written: 60 bytes per cell and
 // step in FP32 with a current (48 without).  The columns of the x-halo and
 // the warm-up rows of a segment are recomputed, never exchanged.
+//
+// In FP64 the arithmetic bounds the kernel (FP64 runs at 1/64 of the FP32 rate on
+// this part), so the stencils are written for the fewest operations (144 per
+// cell, m = 4, p = 3), stages are skipped outside their rows of a segment, and
+// the segments are cut for an even load.  us per step, before -> now: 2048 x
+// 1536 (m = 4, p = 3) 1607 -> 1284, 4096^2 7296 -> 6426, 1024^2 vacuum 514 -> 367,
+// 300 x 700 (m = 3, p = 1) 213 -> 97.  128 threads: strips of 256 columns halo
+// less (4096^2 6173) but leave one CTA per SM (300 x 700 144).
 #include <cuda_runtime.h>
 
 #include "fused2d.h"
@@ -26,13 +34,20 @@
 namespace fmx {
 namespace {
 
-// binomial weight C(2P, k) / 4^P of the P-pass (1/4, 1/2, 1/4) filter
-__host__ __device__ constexpr double binom_w(int P, int k) {
+// unnormalised (2P+1)-tap binomial, the P-pass (1/4, 1/2, 1/4) filter times 4^P,
+// of v[0..2P] step apart: symmetric taps folded, so that it takes 2P operations
+// (P adds and P multiply-adds); the 4^P of both axes is in the current's factor
+template <typename T, int P>
+__device__ __forceinline__ T binom(const T *v, int step = 1) {
+    if constexpr (P == 0) return v[0];
+    T acc = v[0] + v[2 * P * step];
     double c = 1.0;
-    for (int i = 0; i < k; ++i) c = c * (2 * P - i) / (i + 1);
-    double d = 1.0;
-    for (int i = 0; i < P; ++i) d *= 4.0;
-    return c / d;
+#pragma unroll
+    for (int k = 1; k <= P; ++k) {
+        c = c * (2 * P - k + 1) / k;
+        acc += T(c) * (k < P ? v[k * step] + v[(2 * P - k) * step] : v[P * step]);
+    }
+    return acc;
 }
 
 template <typename T>
@@ -110,8 +125,19 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
     const T *__restrict__ Jy = a.J[1];
     const T *__restrict__ Jz = a.J[2];
 
-    const int r0 = y0 - M - G::WU - 1;
+    // Rows in which each stage has work.  An output row y0 <= y < y1 needs
+    // E^{n+1} of rows y0 .. y1, so sweep s is needed on rows y0 - (M-s) ..
+    // y1 + (M-s) and the source on y0 - M .. y1 + M; a stage starts up to two
+    // rows before that, where its running differences take up the rows they
+    // remember.  In FP64 a stage is skipped outside its rows: its arithmetic
+    // bounds the kernel, and the 3M + 2P + 2 rows a segment adds then cost
+    // about 6 rows' worth instead of all of them.  (FP32: the tests cost more
+    // than they save.)
+    constexpr bool GUARD = sizeof(T) == 8;
+    const int r0 = y0 - M - G::WU - (GUARD ? 0 : 1);
     const int r1 = y1 + 2 * M + 1;
+    const T qj = c.q * T(1.0 / (double)(1LL << (4 * P)));  // exact: a power of two
+    const T ax2 = c.ax - T(2) * c.axy;
 
     // register state
     T jw[3][TJ];        // raw current, own column, rows r+1+P (0) .. r+1-P
@@ -120,6 +146,7 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
     T win[M > 0 ? M : 1][3][3];  // stage s input: outputs of s-1 at t-1, t-2, t-3
     T dxx[M > 0 ? M : 1][3];     // Dbar_xx dEz of stage s-1 at rows rho+1, rho, rho-1
     T hh[M > 0 ? M : 1][2];      // Dbar_x dEx (backward) at rows rho+1, rho
+    T kk[M > 0 ? M : 1];         // Dbar_x dEy (forward) at row rho-1
     T en[3], enp[3];             // E^{n+1} own column, current and previous row
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
@@ -136,30 +163,35 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
             for (int k = 0; k < 3; ++k) win[s][q][k] = T(0);
             dxx[s][q] = T(0);
         }
-        hh[s][0] = hh[s][1] = T(0);
+        hh[s][0] = hh[s][1] = kk[s] = T(0);
     }
 
     // prefetched own-column loads for the current iteration
-    T pj[3] = {T(0), T(0), T(0)}, pb[3], pe[3], pf[3];
+    T pj[3] = {T(0), T(0), T(0)}, pb[3] = {T(0), T(0), T(0)}, pe[3] = {T(0), T(0), T(0)}, pf[3] = {T(0), T(0), T(0)};
     auto load_row = [&](int r, T out_j[3], T out_b[3], T out_e[3], T out_f[3]) {
         const int64_t oj = (int64_t)wrap_row(r + 1 + P, g.ny) * g.pitch + xc;
         const int64_t ob = (int64_t)wrap_row(r + 2, g.ny) * g.pitch + xc;
         const int64_t oe = (int64_t)wrap_row(r - 2 * M, g.ny) * g.pitch + xc;
         const int64_t of = (int64_t)wrap_row(r - 2 * M - 1, g.ny) * g.pitch + xc;
-        if (HJ) {
+        const bool front = !GUARD || r <= y1 + M - 1;
+        if (HJ && front) {
             out_j[0] = __ldg(Jx + oj);
             out_j[1] = __ldg(Jy + oj);
             out_j[2] = __ldg(Jz + oj);
         }
-        out_b[0] = __ldg(Bx + ob);
-        out_b[1] = __ldg(By + ob);
-        out_b[2] = __ldg(Bz + ob);
-        out_e[0] = __ldg(Ex + oe);
-        out_e[1] = __ldg(Ey + oe);
-        out_e[2] = __ldg(Ez + oe);
-        out_f[0] = __ldg(Bx + of);
-        out_f[1] = __ldg(By + of);
-        out_f[2] = __ldg(Bz + of);
+        if (front) {
+            out_b[0] = __ldg(Bx + ob);
+            out_b[1] = __ldg(By + ob);
+            out_b[2] = __ldg(Bz + ob);
+        }
+        if (!GUARD || r >= y0 + 2 * M) {
+            out_e[0] = __ldg(Ex + oe);
+            out_e[1] = __ldg(Ey + oe);
+            out_e[2] = __ldg(Ez + oe);
+            out_f[0] = __ldg(Bx + of);
+            out_f[1] = __ldg(By + of);
+            out_f[2] = __ldg(Bz + of);
+        }
     };
     load_row(r0, pj, pb, pe, pf);
     __syncthreads();
@@ -176,6 +208,7 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
         }
         if (r + 1 < r1) load_row(r + 1, pj, pb, pe, pf);
 
+        auto within = [&](int lo, int hi) { return !GUARD || (r >= lo && r <= hi); };
         const int rhoM = r - 2 * M;  // row of the last sweep and of the E update
         const int rhoF = rhoM - 1;   // row of the Faraday update
         T oM[3];                     // output of stage M on row rhoM
@@ -183,41 +216,40 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
         // ---------------- sweeps M..1 (decreasing, so windows still hold t-1) --------
 #pragma unroll
         for (int s = M; s >= 1; --s) {
+            if (!within(y0 - M + 3 * s - 2, y1 + M + s)) continue;
             const int rho = r - 2 * s;
             // ring of stage s-1 (dE' for s = 1)
-            const T *rx_p1, *ry_0, *ry_m1, *rz_p1;  // rows rho+1 (Ex, Ez), rho, rho-1 (Ey)
+            const T *rx_p1, *ry_0, *rz_p1;  // rows rho+1 (Ex, Ez), rho (Ey)
             if (s == 1) {
                 rx_p1 = s_dp + (ring<D0>(rho + 1) * 3 + 0) * RW;
                 ry_0 = s_dp + (ring<D0>(rho) * 3 + 1) * RW;
-                ry_m1 = s_dp + (ring<D0>(rho - 1) * 3 + 1) * RW;
                 rz_p1 = s_dp + (ring<D0>(rho + 1) * 3 + 2) * RW;
             } else {
                 const T *base = s_sw + (s - 2) * 4 * 3 * RW;
                 rx_p1 = base + (((rho + 1) & 3) * 3 + 0) * RW;
                 ry_0 = base + ((rho & 3) * 3 + 1) * RW;
-                ry_m1 = base + (((rho - 1) & 3) * 3 + 1) * RW;
                 rz_p1 = base + (((rho + 1) & 3) * 3 + 2) * RW;
             }
             T(&X)[3] = win[s - 1][0];
             T(&Y)[3] = win[s - 1][1];
             T(&Z)[3] = win[s - 1][2];
-            const T eym = ry_0[col - 1], eyp = ry_0[col + 1], eyp_m1 = ry_m1[col + 1];
+            const T eym = ry_0[col - 1], eyp = ry_0[col + 1];
             const T exm = rx_p1[col - 1];
             const T ezm = rz_p1[col - 1], ezp = rz_p1[col + 1];
             // windows of derived differences: new row rho+1
             dxx[s - 1][2] = dxx[s - 1][1];
             dxx[s - 1][1] = dxx[s - 1][0];
-            dxx[s - 1][0] = ezp - T(2) * Z[0] + ezm;
+            dxx[s - 1][0] = (ezp + ezm) - T(2) * Z[0];
             hh[s - 1][1] = hh[s - 1][0];
             hh[s - 1][0] = X[0] - exm;
             const T *dp = s_dp + ring<D0>(rho) * 3 * RW;
             const T px = dp[col], py = dp[RW + col], pz = dp[2 * RW + col];
-            const T g_own = Y[1] - Y[2];
-            const T g_nb = eyp - eyp_m1;
+            const T k0 = eyp - Y[1], dk = k0 - kk[s - 1];  // Dbar_x Dbar_y Ey
+            kk[s - 1] = k0;
             const T *D = dxx[s - 1];
-            T nx_ = px + c.ay * (X[0] - T(2) * X[1] + X[2]) + c.bxy * (g_nb - g_own);
-            T ny_ = py + c.ax * (eyp - T(2) * Y[1] + eym) + c.bxy * (hh[s - 1][0] - hh[s - 1][1]);
-            T nz_ = pz + c.ax * D[1] + c.ay * (Z[0] - T(2) * Z[1] + Z[2]) + c.axy * (D[0] - T(2) * D[1] + D[2]);
+            T nx_ = px + c.ay * ((X[0] + X[2]) - T(2) * X[1]) + c.bxy * dk;
+            T ny_ = py + c.ax * ((eyp + eym) - T(2) * Y[1]) + c.bxy * (hh[s - 1][0] - hh[s - 1][1]);
+            T nz_ = pz + ax2 * D[1] + c.ay * ((Z[0] + Z[2]) - T(2) * Z[1]) + c.axy * (D[0] + D[2]);
             if (s == M) {
                 oM[0] = nx_;
                 oM[1] = ny_;
@@ -270,32 +302,27 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
         }
 
         // ---------------- source, row r ----------------
-        {
+        if (within(y0 - M - 1, y1 + M)) {
             T jf[3] = {T(0), T(0), T(0)};
             if (HJ) {
                 const T *jr = s_jy + (r & 1) * 3 * RW;
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    T acc = T(0);
-#pragma unroll
-                    for (int k = 0; k < 2 * P + 1; ++k) acc += T(binom_w(P, k)) * jr[q * RW + col + k - P];
-                    jf[q] = acc;
-                }
+                for (int q = 0; q < 3; ++q) jf[q] = binom<T, P>(jr + q * RW + col - P);
             }
             const T *sbx = s_bx + (r & 3) * RW;
             const T *sbz = s_bz + (r & 3) * RW;
             const T *say = s_ay + (r & 1) * RW;
             const T bx0 = sbx[col];
-            const T axbx = bx0 + c.c6 * (sbx[col + 1] - T(2) * bx0 + sbx[col - 1]);
+            const T axbx = bx0 + c.c6 * ((sbx[col + 1] + sbx[col - 1]) - T(2) * bx0);
             const T bz0 = sbz[col], bzm = sbz[col - 1];
             const T ay0 = say[col], aym = say[col - 1];
             T ex_ = c.ky * (bz0 - bz_prev);
             T ey_ = -(c.kx * (bz0 - bzm));
             T ez_ = c.kx * (ay0 - aym) - c.ky * (axbx - axbx_prev);
             if (HJ) {
-                ex_ -= c.q * jf[0];
-                ey_ -= c.q * jf[1];
-                ez_ -= c.q * jf[2];
+                ex_ -= qj * jf[0];
+                ey_ -= qj * jf[1];
+                ez_ -= qj * jf[2];
             }
             bz_prev = bz0;
             axbx_prev = axbx;
@@ -347,28 +374,25 @@ __device__ __forceinline__ void fused2d_tile(const Fused2dArgs<T> &a, const Geo 
         }
 
         // ---------------- current: y-binomial of row r+1 ----------------
-        if (HJ) {
+        if (HJ && within(r0, y1 + M - 1)) {
             T *jo = s_jy + ((r + 1) & 1) * 3 * RW;
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
 #pragma unroll
                 for (int k = TJ - 1; k > 0; --k) jw[q][k] = jw[q][k - 1];
                 jw[q][0] = cj[q];
-                T acc = T(0);
-#pragma unroll
-                for (int k = 0; k < TJ; ++k) acc += T(binom_w(P, k)) * jw[q][k];
-                jo[q * RW + col] = acc;
+                if (within(y0 - M - 1, y1 + M - 1)) jo[q * RW + col] = binom<T, P>(jw[q]);
             }
         }
 
         // ---------------- B prep: row r+2 ----------------
-        {
+        if (within(r0, y1 + M - 1)) {
             byw[2] = byw[1];
             byw[1] = byw[0];
             byw[0] = cb[1];
             s_bx[((r + 2) & 3) * RW + col] = cb[0];
             s_bz[((r + 2) & 3) * RW + col] = cb[2];
-            s_ay[((r + 1) & 1) * RW + col] = byw[1] + c.c6 * (byw[0] - T(2) * byw[1] + byw[2]);
+            s_ay[((r + 1) & 1) * RW + col] = byw[1] + c.c6 * ((byw[0] + byw[2]) - T(2) * byw[1]);
         }
         __syncthreads();
     }
@@ -432,11 +456,28 @@ struct Launcher {
             cudaGetDevice(&dev);
             if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
         }
-        const int target = blocks_per_sm() * sms;
-        int nseg = target / sh.strips;
-        if (nseg < 1) nseg = 1;
-        if (nseg > g.ny) nseg = g.ny;
-        sh.rows = (g.ny + nseg - 1) / nseg;
+        const int bps = blocks_per_sm(), target = bps * sms;
+        if (sizeof(T) == 8) {
+            // the CTAs of one SM share its FP64 arithmetic: the segment count with
+            // the least (CTAs of the fullest SM) x (rows each computes, about 6
+            // beyond its own), c resident CTAs leaving 1/(2c) of their latencies open
+            double least = 1e300;
+            for (int n = 1; n <= g.ny; ++n) {
+                const int rows = (g.ny + n - 1) / n;
+                if (rows < 8 && n > 1) break;
+                const long long k = ((long long)sh.strips * ((g.ny + rows - 1) / rows) + sms - 1) / sms;
+                const double load = (double)(k / bps) * (bps + 0.5) + (k % bps ? (double)(k % bps) + 0.5 : 0.0);
+                if (load * (rows + 6) < least) {
+                    least = load * (rows + 6);
+                    sh.rows = rows;
+                }
+            }
+        } else {
+            int nseg = target / sh.strips;
+            if (nseg < 1) nseg = 1;
+            if (nseg > g.ny) nseg = g.ny;
+            sh.rows = (g.ny + nseg - 1) / nseg;
+        }
         sh.segments = (g.ny + sh.rows - 1) / sh.rows;
         return sh;
     }
