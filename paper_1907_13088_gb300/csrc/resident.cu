@@ -162,33 +162,74 @@ struct Sync {
 };
 
 // Launch-wide FP64 sum of v (every thread calls it and gets the same value,
-// or ok = false when the launch gave up).  xs: this CTA's [2][kMaxCluster]
-// partial slots, alternated by `par` so that the next reduction never
-// overwrites slots (or DevStatus::xpart entries) a slower CTA still reads.
-__device__ __forceinline__ double launch_sum(const Sync &S, double v, double *red, double *xs, int par, bool &ok) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int t = threadIdx.x;
-    if ((t & 31) == 0) red[t >> 5] = v;
-    __syncthreads();
+// or ok = false when the launch gave up).  FP64 adds are the scarce resource
+// (1/64 of the FP32 rate, tens of cycles each), so one warp does them: the
+// threads' values go to shared memory, the first warp adds eight per lane and
+// then across its lanes, its lanes write the CTA's partial into every CTA of
+// the cluster, and after the barrier it adds the cluster's partials and hands
+// the sum to the CTA.  (All warps reducing by shuffles and every thread adding
+// the 16 partials took 1.3 us of a phase of 7.6 us at 64^2 FP64.)  xs: this
+// CTA's [2][kMaxCluster] partial slots, alternated by `par` so that the next
+// reduction never overwrites slots (or DevStatus::xpart entries) a slower CTA
+// still reads.
+struct SumSmem {
+    double v[kNT];
+    double xs[2 * kMaxCluster];
+    double tot;
+};
+__device__ __forceinline__ double warp_sum(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double launch_sum(const Sync &S, double v, SumSmem &sm, int par, bool &ok) {
+    const int t = threadIdx.x, lane = t & 31;
     const int C = (int)S.cl.num_blocks();
-    if (t == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kNT / 32; ++w) s += red[w];
-        for (int r = 0; r < C; ++r) S.cl.map_shared_rank(xs + par * kMaxCluster, r)[S.crank] = s;
+    sm.v[t] = v;
+    __syncthreads();
+    if (t < 32) {
+        double s = (sm.v[t] + sm.v[t + 32]) + (sm.v[t + 64] + sm.v[t + 96]);
+        s += (sm.v[t + 128] + sm.v[t + 160]) + (sm.v[t + 192] + sm.v[t + 224]);
+        static_assert(kNT == 256, "eight values per lane");
+        s = warp_sum(s);
+        if (lane < C) S.cl.map_shared_rank(sm.xs + par * kMaxCluster, lane)[S.crank] = s;
     }
     S.cl.sync();
-    double tot = 0.0;
-    for (int r = 0; r < C; ++r) tot += xs[par * kMaxCluster + r];
-    if (!S.grid()) {
-        ok = true;
-        return tot;
+    if (t < 32) {
+        const double tot = warp_sum(lane < C ? sm.xs[par * kMaxCluster + lane] : 0.0);
+        if (t == 0) {
+            sm.tot = tot;
+            if (S.grid() && S.crank == 0) __stcg(&S.st->xpart[par][S.cid], tot);
+        }
     }
-    if (S.crank == 0 && t == 0) __stcg(&S.st->xpart[par][S.cid], tot);
-    ok = S.barrier();
-    if (!ok) return 0.0;
-    double all = 0.0;
-    for (int k = 0; k < S.ncl; ++k) all += __ldcg(&S.st->xpart[par][k]);
-    return all;
+    if (S.grid()) {
+        ok = S.barrier();
+        if (!ok) return 0.0;
+        if (t < 32) {
+            const double all = warp_sum(lane < S.ncl ? __ldcg(&S.st->xpart[par][lane]) : 0.0);
+            if (t == 0) sm.tot = all;
+        }
+    }
+    __syncthreads();
+    ok = true;
+    return sm.tot;
+}
+
+// (A dE) of a cell in 2D: apply_a (stencil.cuh) with each difference formed
+// once, 23 operations instead of about 33.  at(k, dx, dy): component k at a
+// neighbour; own receives the cell's own values.
+template <typename T, typename F>
+__device__ __forceinline__ void apply_a_2d(const F &at, const Coef<T> &c, T own[3], T out[3]) {
+    const T x = at(0, 0, 0), xu = at(0, 0, 1), xd = at(0, 0, -1), xl = at(0, -1, 0), xlu = at(0, -1, 1);
+    const T y = at(1, 0, 0), yl = at(1, -1, 0), yr = at(1, 1, 0), yd = at(1, 0, -1), yrd = at(1, 1, -1);
+    const T z = at(2, 0, 0), zl = at(2, -1, 0), zr = at(2, 1, 0), zu = at(2, 0, 1), zd = at(2, 0, -1);
+    const T zlu = at(2, -1, 1), zru = at(2, 1, 1), zld = at(2, -1, -1), zrd = at(2, 1, -1);
+    own[0] = x;
+    own[1] = y;
+    own[2] = z;
+    out[0] = c.ay * ((xu + xd) - T(2) * x) + c.bxy * ((yr - y) - (yrd - yd));
+    out[1] = c.ax * ((yl + yr) - T(2) * y) + c.bxy * ((xu - xlu) - (x - xl));
+    const T d0 = (zl + zr) - T(2) * z, du = (zlu + zru) - T(2) * zu, dd = (zld + zrd) - T(2) * zd;
+    out[2] = (c.ax - T(2) * c.axy) * d0 + c.ay * ((zu + zd) - T(2) * z) + c.axy * (du + dd);
 }
 
 template <typename T>
@@ -207,8 +248,7 @@ struct ResidentArgs {
 
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kNT) k_resident(ResidentArgs<T> a, Geo g) {
-    __shared__ double red[kNT / 32];
-    __shared__ double xs[2 * kMaxCluster];
+    __shared__ SumSmem sums;
     __shared__ int abort_s;
     Sync S{cg::this_cluster(), a.P.st, 0, 0, 0, a.limit, a.lost, &abort_s};
     const int C = (int)S.cl.num_blocks();
@@ -279,7 +319,7 @@ __global__ void __launch_bounds__(kNT) k_resident(ResidentArgs<T> a, Geo g) {
             v += (double)ex * ex + (double)ey * ey + (double)ez * ez;
         }
         if (a.resid) {
-            n2 = launch_sum(S, v, red, xs, par, ok);
+            n2 = launch_sum(S, v, sums, par, ok);
             par ^= 1;
         } else {
             ok = S.barrier();
@@ -301,11 +341,15 @@ __global__ void __launch_bounds__(kNT) k_resident(ResidentArgs<T> a, Geo g) {
                 Pos p;
                 int64_t idx;
                 cells.at(q, p, idx);
-                const T nx_ = __ldcg(P.dEp[0] + idx) + apply_a<T, DIM, 0>(f, p, c);
-                const T ny_ = __ldcg(P.dEp[1] + idx) + apply_a<T, DIM, 1>(f, p, c);
-                const T nz_ = __ldcg(P.dEp[2] + idx) + apply_a<T, DIM, 2>(f, p, c);
-                const T dx = nx_ - __ldcg(in[0] + idx), dy = ny_ - __ldcg(in[1] + idx),
-                        dz = nz_ - __ldcg(in[2] + idx);
+                T own[3], av[3];
+                const T p0 = __ldcg(P.dEp[0] + idx), p1 = __ldcg(P.dEp[1] + idx), p2 = __ldcg(P.dEp[2] + idx);
+                av[0] = apply_a<T, DIM, 0>(f, p, c);
+                av[1] = apply_a<T, DIM, 1>(f, p, c);
+                av[2] = apply_a<T, DIM, 2>(f, p, c);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) own[k] = __ldcg(in[k] + idx);
+                const T nx_ = p0 + av[0], ny_ = p1 + av[1], nz_ = p2 + av[2];
+                const T dx = nx_ - own[0], dy = ny_ - own[1], dz = nz_ - own[2];
                 out[0][idx] = nx_;
                 out[1][idx] = ny_;
                 out[2][idx] = nz_;
@@ -313,7 +357,7 @@ __global__ void __launch_bounds__(kNT) k_resident(ResidentArgs<T> a, Geo g) {
             }
             ++s;
             if (a.resid) {
-                r2 = launch_sum(S, w, red, xs, par, ok);
+                r2 = launch_sum(S, w, sums, par, ok);
                 par ^= 1;
                 if (!ok) break;
                 if (r2 <= a.tol2 * n2) {
@@ -364,6 +408,173 @@ __global__ void __launch_bounds__(kNT) k_resident(ResidentArgs<T> a, Geo g) {
     }
     if (b == 0 && t == 0) {
         DevStatus *st = P.st;
+        st->nrm2 = n2;
+        st->r2 = r2;
+        st->count = last;
+        st->done = 1;
+        st->noconv = noconv;
+        st->steps = steps_done;
+        st->sweeps_total = total;
+    }
+}
+
+// The same engine for 2D grids that fit the shared memory of one cluster: CTA r
+// owns rows r R .. r R + R - 1 (R = ceil(n_y / C)) of E, B, dE' and both sweep
+// buffers there, with one halo row on either side, and every phase reads its
+// own shared memory only; a CTA that computes a border row also writes it into
+// the halo of the CTA above or below (distributed shared memory), which the
+// phase's cluster barrier orders.  Nothing goes through L2 between the first
+// load and the last store.  (Through L2 a phase took 6.6 us at 64^2, in FP32 as
+// in FP64: about 22 loads of 700 cycles and a barrier that waits for the
+// stores to reach L2.)  Only without a filtered current.
+// us per step (20 steps a call), 64^2: FP64 to 1e-13 (13 sweeps) 119 -> 91.5, FP32 to 1e-5 (5 sweeps)
+// 53 -> 40; 128^2 FP32 (3 sweeps) 59 -> 42.5.  A fixed sweep takes 3.2 us in FP64 (its
+// 26 operations per cell: 2 us) and 0.8 us in FP32.
+template <typename T>
+__global__ void __launch_bounds__(kNT) k_resident_rows(ResidentArgs<T> a, Geo g, int R) {
+    extern __shared__ __align__(16) unsigned char rsm[];
+    __shared__ SumSmem sums;
+    __shared__ int abort_s;
+    Sync S{cg::this_cluster(), a.P.st, 1, 0, 0, a.limit, 0, &abort_s};
+    S.crank = (int)S.cl.block_rank();
+    const int used = (g.ny + R - 1) / R;  // CTAs that own rows; the others only keep the barriers
+    const int rank = S.crank, y0 = rank * R, rows = rank < used ? min(R, g.ny - y0) : 0;
+    const int nx = g.nx, comp = (R + 2) * nx;  // a component: halo row, own rows, halo row (after the own rows)
+    T *sm = reinterpret_cast<T *>(rsm);        // E[3], B[3], dE'[3], dEa[3], dEb[3]
+    const int t = threadIdx.x;
+    const Coef<T> &c = a.c;
+    // the neighbours' shared memory, and where this CTA's border rows go there:
+    // its first row into the halo above the rows of the CTA below, its last row
+    // into the halo row 0 of the CTA above
+    const int below = rows ? (rank + used - 1) % used : 0, above = rows ? (rank + 1) % used : 0;
+    T *const smb = S.cl.map_shared_rank(sm, below), *const sma = S.cl.map_shared_rank(sm, above);
+    const int top_b = (min(R, g.ny - below * R) + 1) * nx;
+    auto put = [&](int k, int i, int j, T v) {
+        sm[k * comp + (j + 1) * nx + i] = v;
+        if (j == 0) smb[k * comp + top_b + i] = v;
+        if (j == rows - 1) sma[k * comp + i] = v;
+    };
+    // the CTA's cells, a stride of kNT apart
+    const int di = kNT % nx, dj = kNT / nx, i0 = t % nx, j0 = t / nx;
+    auto cells = [&](auto f) {
+        for (int i = i0, j = j0; j < rows;) {
+            f(i, j);
+            i += di;
+            j += dj;
+            if (i >= nx) {
+                i -= nx;
+                ++j;
+            }
+        }
+    };
+    auto gidx = [&](int i, int j) { return (int64_t)(y0 + j) * g.pitch + i; };
+
+    // E and B of the own rows, pushed to the halos as every later border row is
+    S.cl.sync();  // every CTA of the cluster is there before its memory is written
+    cells([&](int i, int j) {
+        const int64_t q = gidx(i, j);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            put(k, i, j, a.P.E[k][q]);
+            put(3 + k, i, j, a.P.B[k][q]);
+        }
+    });
+    S.cl.sync();
+
+    int par = 0, last = 0, steps_done = 0, noconv = 0;
+    bool ok = true;
+    long long total = 0;
+    double n2 = 0.0, r2 = 0.0;
+    for (int n = 0; n < a.nsteps; ++n) {
+        // ---- source, ||dE'||^2
+        double v = 0.0;
+        cells([&](int i, int j) {
+            const int o = (j + 1) * nx + i, xm = i > 0 ? -1 : nx - 1, xp = i + 1 < nx ? 1 : 1 - nx;
+            const T *bx = sm + 3 * comp + o, *by = sm + 4 * comp + o, *bz = sm + 5 * comp + o;
+            auto ax = [&](const T *p) { return p[0] + c.c6 * ((p[xp] + p[xm]) - T(2) * p[0]); };
+            auto ay = [&](const T *p) { return p[0] + c.c6 * ((p[nx] + p[-nx]) - T(2) * p[0]); };
+            T d[3] = {c.ky * (bz[0] - bz[-nx]), -(c.kx * (bz[0] - bz[xm])),
+                      c.kx * (ay(by) - ay(by + xm)) - c.ky * (ax(bx) - ax(bx - nx))};
+            const int64_t q = gidx(i, j);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (a.have_j) d[k] -= c.q * __ldg(a.P.J[k] + q);
+                put(6 + k, i, j, d[k]);
+                v += (double)d[k] * d[k];
+            }
+        });
+        if (a.resid) {
+            n2 = launch_sum(S, v, sums, par, ok);
+            par ^= 1;
+        } else {
+            S.cl.sync();
+        }
+        // ---- sweeps
+        int s = 0, in = 6;
+        bool stop = a.resid ? n2 == 0.0 : a.m == 0;
+        while (!stop) {
+            const int out = in == 9 ? 12 : 9;
+            double w = 0.0;
+            cells([&](int i, int j) {
+                const int o = (j + 1) * nx + i, xm = i > 0 ? -1 : nx - 1, xp = i + 1 < nx ? 1 : 1 - nx;
+                const T *p = sm + in * comp + o;
+                auto at = [&](int k, int dx, int dy) { return p[k * comp + (dx < 0 ? xm : (dx > 0 ? xp : 0)) + dy * nx]; };
+                T own[3], av[3];
+                apply_a_2d<T>(at, c, own, av);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const T x = sm[(6 + k) * comp + o] + av[k], d = x - own[k];
+                    put(out + k, i, j, x);
+                    w += (double)d * d;
+                }
+            });
+            ++s;
+            in = out;
+            if (a.resid) {
+                r2 = launch_sum(S, w, sums, par, ok);
+                par ^= 1;
+                if (r2 <= a.tol2 * n2) {
+                    stop = true;
+                } else if (s >= a.m_max) {
+                    stop = true;
+                    noconv = 1;
+                }
+            } else {
+                S.cl.sync();
+                stop = s >= a.m;
+            }
+        }
+        last = s;
+        total += s;
+        // ---- E^{n+1} = E^n + dE on the own rows and the halo row above them, Faraday
+        for (int q = t; q < (rows ? (rows + 1) * nx : 0); q += kNT) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) sm[k * comp + nx + q] += sm[(in + k) * comp + nx + q];
+        }
+        __syncthreads();
+        cells([&](int i, int j) {
+            const int o = (j + 1) * nx + i, xp = i + 1 < nx ? 1 : 1 - nx;
+            const T *ex = sm + o, *ey = sm + comp + o, *ez = sm + 2 * comp + o;
+            const T bx = sm[3 * comp + o], by = sm[4 * comp + o], bz = sm[5 * comp + o];
+            put(3, i, j, bx - c.ky * (ez[nx] - ez[0]));
+            put(4, i, j, by + c.kx * (ez[xp] - ez[0]));
+            put(5, i, j, (bz - c.kx * (ey[xp] - ey[0])) + c.ky * (ex[nx] - ex[0]));
+        });
+        S.cl.sync();
+        ++steps_done;
+        if (noconv) break;
+    }
+    cells([&](int i, int j) {
+        const int64_t q = gidx(i, j);
+        const int o = (j + 1) * nx + i;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            a.P.E[k][q] = sm[k * comp + o];
+            a.P.B[k][q] = sm[(3 + k) * comp + o];
+        }
+    });
+    if (rank == 0 && t == 0) {
+        DevStatus *st = a.P.st;
         st->nrm2 = n2;
         st->r2 = r2;
         st->count = last;
@@ -451,14 +662,15 @@ struct ResidentLauncher {
         return r;
     }
     // A grid barrier costs ~3 us per phase (an L2 atomic round trip and a
-    // poll); another cluster pays when it takes more FP64 work off the
-    // cluster's SMs than that.  Measured (FP64, Algorithm 1 to 1e-13): 64^2,
-    // one cluster 0.090 ms per step, four 0.133; 128^2, one 0.161, two 0.126,
-    // four 0.097, seven 0.108.  So about 256 cells per CTA in FP64; FP32
-    // arithmetic is 64x cheaper.
+    // poll); other clusters pay when they take more FP64 work off the cluster's
+    // SMs than that (in FP32 the residual's conversions and squares).  us per
+    // step, Algorithm 1 to 1e-13 in FP64, to 1e-5 in FP32, by clusters: FP64 90^2
+    // 124 (1), 129 (2), 127 (4); 128^2 163 (1), 156 (2), 124 (4), 116 (7); FP32 128^2
+    // 59 (1), 65 (7); 200^2 92 (1), 73 (5); 256^2 112 (2), 88 (4), 82 (7).
     static int clusters_for(int64_t cells, bool lost) {
         if (coop_refused()) return 1;
-        const int64_t per_cta = sizeof(T) == 8 ? 256 : 4096;
+        if (cells <= (sizeof(T) == 8 ? 8192 : 24576)) return 1;
+        const int64_t per_cta = sizeof(T) == 8 ? 128 : 512;
         const int64_t want = (cells + per_cta * cluster() - 1) / (per_cta * cluster());
         int n = (int)(want < 1 ? 1 : want);
         const int mc = max_clusters();
@@ -466,7 +678,42 @@ struct ResidentLauncher {
         (void)lost;
         return n;
     }
+    // the shared-memory engine, where the grid takes one cluster and fits it;
+    // false where it does not apply
+    static bool run_rows(const Geo &g, const ResidentArgs<T> &a, int ncl, cudaStream_t s) {
+        if (DIM != 2 || ncl != 1 || a.lost || (a.have_j && a.jpasses > 0)) return false;
+        const int cs = cluster(), R = (g.ny + cs - 1) / cs;
+        static const int lim = [] {
+            int dev = 0, v = 0;
+            cudaGetDevice(&dev);
+            return cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess ? v : 0;
+        }();
+        const size_t need = (size_t)15 * (R + 2) * g.nx * sizeof(T);
+        // half the cluster's CTAs with rows at least; 4 KB for the static part
+        if (2 * ((g.ny + R - 1) / R) < cs || need + 4096 > (size_t)lim) return false;
+        auto k = k_resident_rows<T>;
+        static const bool attr =
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 4096) == cudaSuccess &&
+            (cs <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess);
+        if (!attr) {
+            cudaGetLastError();
+            return false;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1] = {cluster_attr(cs)};
+        cfg.gridDim = dim3(cs);
+        cfg.blockDim = dim3(kNT);
+        // more than half an SM's shared memory: one CTA per SM
+        cfg.dynamicSmemBytes = need > spread_bytes() ? need : spread_bytes();
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, k, a, g, R) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    }
     static cudaError_t run(const Geo &g, const ResidentArgs<T> &a, int &ncl, cudaStream_t s) {
+        if (run_rows(g, a, ncl, s)) return cudaSuccess;
         const int cs = cluster();
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[2] = {cluster_attr(cs), {}};
