@@ -58,9 +58,13 @@ class GaussSourceRun:
 
     # ------------------------------------------------------------------
     def _state(self):
-        out = self.torch.empty((9, 1) + self.shape[::-1], dtype=self.grid.dtype, device=self.grid.device)
-        E, B, _ = self.grid.get_fields(fmx.FMX_E | fmx.FMX_B, out=out)
-        return E[:, 0].clone(), B[:, 0].clone()
+        """A copy of the grid's state, (E, B) of shape (3, ny, nx) each."""
+        g = self.grid
+        out = self.torch.empty((6,) + self.shape[::-1], dtype=g.dtype, device=g.device)
+        csz = g.cells * out.element_size()
+        ptrs = (ctypes.c_void_p * 9)(*[out.data_ptr() + c * csz for c in range(6)], None, None, None)
+        fmx.check(fmx.fmx_get_fields(g.handle, fmx.FMX_E | fmx.FMX_B, ptrs, fmx.FMX_DEVICE), "fmx_get_fields")
+        return out[:3], out[3:]
 
     def _setup(self, theta):
         th = np.ascontiguousarray(np.asarray(theta, dtype=np.float64))

@@ -10,8 +10,9 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <new>
 #include <algorithm>
+#include <atomic>
+#include <new>
 #include <map>
 #include <mutex>
 #include <string>
@@ -587,6 +588,19 @@ fmx_status staged_step(fmx_grid *g) {
     return FMX_OK;
 }
 
+// SM clock rate of the current device in kHz, asked for once per device: the
+// query goes to the driver and takes about 450 us
+int sm_clock_khz() {
+    static std::atomic<int> cache[64];
+    int dev = 0, khz = 0;
+    cudaGetDevice(&dev);
+    const bool in = dev >= 0 && dev < 64;
+    if (in && (khz = cache[dev].load(std::memory_order_relaxed)) > 0) return khz;
+    if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) khz = 2000000;
+    if (in) cache[dev].store(khz, std::memory_order_relaxed);
+    return khz;
+}
+
 // Resident engine: nsteps steps in one launch (one cluster, or several in a
 // cooperative launch).  The status word is cleared first (arrival count,
 // generation, latched error).  Residual mode, and any launch over several
@@ -601,9 +615,7 @@ fmx_status resident_steps(fmx_grid *g, int nsteps) {
     const bool resid = g->p.iter_mode == FMX_ITER_RESIDUAL;
     const bool have_j = g->buf.J[0] != nullptr;
     const int jpasses = (have_j && g->p.filter_target == FMX_FILTER_CURRENT) ? g->p.filter_passes : 0;
-    int dev = 0, khz = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) khz = 2000000;
+    const int khz = sm_clock_khz();
     fmx::ResidentWait wait;
     wait.limit_cycles = (long long)g->wait_limit_us * (long long)khz / 1000;
     wait.lost_arrival = g->lost_arrival;
@@ -754,10 +766,10 @@ fmx_status fused_step(fmx_grid *g, int nsteps, StepPre pre = nullptr) {
 // and the grid's pitched array: one 1D copy when the rows are contiguous on
 // both sides, else a 2D copy; on `stream` (the grid's stream by default).
 fmx_status copy_rows(fmx_grid *g, void *dst, size_t dpitch, const void *src, size_t spitch, bool sync,
-                     cudaStream_t stream = nullptr) {
+                     cudaStream_t stream = nullptr, int ncomp = 1) {
     const cudaStream_t st = stream ? stream : g->stream;
     const size_t width = (size_t)g->geo.nx * g->elem;
-    const size_t rows = (size_t)g->geo.ny * (size_t)g->geo.nz;
+    const size_t rows = (size_t)g->geo.ny * (size_t)g->geo.nz * (size_t)ncomp;
     cudaError_t e;
     if (dpitch == width && spitch == width)
         e = cudaMemcpyAsync(dst, src, width * rows, cudaMemcpyDefault, st);
@@ -767,6 +779,35 @@ fmx_status copy_rows(fmx_grid *g, void *dst, size_t dpitch, const void *src, siz
     if (sync) {
         e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    }
+    return FMX_OK;
+}
+
+// Components in mask (of n pointer pairs), dense on one side and pitched on the
+// other, on the grid's stream: neighbouring components whose arrays follow each
+// other without a gap on both sides go in one copy.
+fmx_status copy_components(fmx_grid *g, int n, unsigned mask, void *const *dst, size_t dpitch, const void *const *src,
+                           size_t spitch) {
+    const size_t rows = (size_t)g->geo.ny * (size_t)g->geo.nz;
+    for (int c = 0; c < n;) {
+        if (!(mask & (1u << c))) {
+            ++c;
+            continue;
+        }
+        int k = 1;
+        while (c + k < n && (mask & (1u << (c + k))) &&
+               (const char *)src[c + k] == (const char *)src[c] + k * rows * spitch &&
+               (char *)dst[c + k] == (char *)dst[c] + k * rows * dpitch)
+            ++k;
+        fmx_status s = copy_rows(g, dst[c], dpitch, src[c], spitch, false, nullptr, k);
+        if (s != FMX_OK && k > 1) {
+            // neighbours by address but not one allocation: each by itself
+            cudaGetLastError();
+            s = FMX_OK;
+            for (int q = c; q < c + k && s == FMX_OK; ++q) s = copy_rows(g, dst[q], dpitch, src[q], spitch, false);
+        }
+        if (s != FMX_OK) return s;
+        c += k;
     }
     return FMX_OK;
 }
@@ -1001,13 +1042,13 @@ fmx_status fmx_set_fields(fmx_grid *g, unsigned mask, const void *const *src, in
     if (!g->bound) return fail(FMX_ESTATE, "grid not bound");
     if (mask & ~(unsigned)(FMX_E | FMX_B)) return fail(FMX_EINVAL, "mask holds bits other than E and B");
     const size_t sp = (size_t)g->geo.nx * g->elem, dp = (size_t)g->geo.pitch * g->elem;
+    void *dst[6];
     for (int c = 0; c < 6; ++c) {
-        if (!(mask & (1u << c))) continue;
-        if (!src[c]) return fail(FMX_EINVAL, "src[%d] is NULL", c);
-        void *dst = c < 3 ? g->buf.E[g->cur][c] : g->buf.B[g->cur][c - 3];
-        fmx_status s = copy_rows(g, dst, dp, src[c], sp, false);
-        if (s != FMX_OK) return s;
+        if ((mask & (1u << c)) && !src[c]) return fail(FMX_EINVAL, "src[%d] is NULL", c);
+        dst[c] = c < 3 ? g->buf.E[g->cur][c] : g->buf.B[g->cur][c - 3];
     }
+    const fmx_status s = copy_components(g, 6, mask, dst, dp, src, sp);
+    if (s != FMX_OK) return s;
     if (where == FMX_HOST) {
         cudaError_t e = cudaStreamSynchronize(g->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
@@ -1033,11 +1074,10 @@ fmx_status fmx_set_current(fmx_grid *g, const void *const *src, int where) {
     if (!g->bound) return fail(FMX_ESTATE, "grid not bound");
     if (!g->buf.J[0]) return fail(FMX_ESTATE, "no J buffers bound");
     const size_t sp = (size_t)g->geo.nx * g->elem, dp = (size_t)g->geo.pitch * g->elem;
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < 3; ++c)
         if (!src[c]) return fail(FMX_EINVAL, "src[%d] is NULL", c);
-        fmx_status s = copy_rows(g, g->buf.J[c], dp, src[c], sp, false);
-        if (s != FMX_OK) return s;
-    }
+    const fmx_status s = copy_components(g, 3, 7u, g->buf.J, dp, src, sp);
+    if (s != FMX_OK) return s;
     if (where == FMX_HOST) {
         cudaError_t e = cudaStreamSynchronize(g->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
@@ -1099,13 +1139,13 @@ fmx_status fmx_get_fields(fmx_grid *g, unsigned mask, void *const *dst, int wher
     if (mask & ~(unsigned)(FMX_E | FMX_B | FMX_J)) return fail(FMX_EINVAL, "bad mask");
     if ((mask & FMX_J) && !g->buf.J[0]) return fail(FMX_ESTATE, "no J buffers bound");
     const size_t dp = (size_t)g->geo.nx * g->elem, sp = (size_t)g->geo.pitch * g->elem;
+    const void *src[9];
     for (int c = 0; c < 9; ++c) {
-        if (!(mask & (1u << c))) continue;
-        if (!dst[c]) return fail(FMX_EINVAL, "dst[%d] is NULL", c);
-        const void *f = c < 3 ? g->buf.E[g->cur][c] : (c < 6 ? g->buf.B[g->cur][c - 3] : g->buf.J[c - 6]);
-        fmx_status s = copy_rows(g, dst[c], dp, f, sp, false);
-        if (s != FMX_OK) return s;
+        if ((mask & (1u << c)) && !dst[c]) return fail(FMX_EINVAL, "dst[%d] is NULL", c);
+        src[c] = c < 3 ? g->buf.E[g->cur][c] : (c < 6 ? g->buf.B[g->cur][c - 3] : g->buf.J[c - 6]);
     }
+    const fmx_status s = copy_components(g, 9, mask, dst, dp, src, sp);
+    if (s != FMX_OK) return s;
     return fmx_sync(g);
 }
 

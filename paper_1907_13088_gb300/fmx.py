@@ -366,7 +366,23 @@ class Grid:
         grid's size, dtype and device)."""
         return component_ptrs(arrays, self.cells, self.np_dtype, self.dtype, self._dev_index, out)
 
+    def _whole_ptr(self, F, ncomp):
+        """Address of a tensor that holds ncomp components back to back, ready to
+        copy (contiguous, this grid's dtype, device and size), or None: the caller
+        then goes through the components one by one, with their checks."""
+        if _is_tensor(F) and F.is_cuda and F.dtype == self.dtype and F.dim() and F.shape[0] == ncomp \
+                and F.numel() == ncomp * self.cells and F.is_contiguous() and F.device.index == self._dev_index:
+            return F.data_ptr()
+        return None
+
     def set_fields(self, E=None, B=None):
+        whole = [None if F is None else self._whole_ptr(F, 3) for F in (E, B)]
+        if all(F is None or p is not None for F, p in zip((E, B), whole)):
+            csz = self.cells * self._slab.element_size()
+            ptrs = (ctypes.c_void_p * 6)(*[None if p is None else p + c * csz for p in whole for c in range(3)])
+            mask = (FMX_E if E is not None else 0) | (FMX_B if B is not None else 0)
+            check(fmx_set_fields(self.handle, mask, ptrs, FMX_DEVICE), "fmx_set_fields")
+            return
         arrs = [None] * 6
         mask = 0
         for k, F in enumerate((E, B)):
@@ -384,6 +400,12 @@ class Grid:
     def set_current(self, J):
         if len(J) != 3:
             raise ValueError(f"J must have 3 components (got {len(J)})")
+        base = self._whole_ptr(J, 3)
+        if base is not None:
+            csz = self.cells * self._slab.element_size()
+            check(fmx_set_current(self.handle, (ctypes.c_void_p * 3)(base, base + csz, base + 2 * csz), FMX_DEVICE),
+                  "fmx_set_current")
+            return
         ptrs, keep, where = self._ptr_array([J[0], J[1], J[2]])
         check(fmx_set_current(self.handle, ptrs, where), "fmx_set_current")
         del keep
