@@ -25,6 +25,11 @@
 #include "pair2.cuh"
 
 namespace fmx {
+
+// the adjoint step of one set on register tiles (adj_tile2d.cu)
+template <int POL, int M, int P, bool HJB>
+void launch_adj_tile2d(const Geo &g, const pair2::Coef2 &c, const Adj2dArgs<float> &a, cudaStream_t s);
+
 namespace {
 
 using namespace pair2;
@@ -423,6 +428,8 @@ __global__ void __launch_bounds__(NT, 3)
 // rows per segment asked for by the caller of the current launch (0:
 // automatic, see AdjLauncher::run)
 thread_local int t_adj_rows = 0;
+// stream of the TE launch (nullptr: the caller's)
+thread_local cudaStream_t t_adj_te = nullptr;
 
 template <int POL, int M, int P, bool HJB>
 struct AdjLauncher {
@@ -441,6 +448,7 @@ struct AdjLauncher {
         return b;
     }
     static void run(const Geo &g, const Coef2 &c, const Adj2dArgs<float> &a, cudaStream_t s) {
+        if (t_adj_rows == 0 && fused2d_tiles(g)) return launch_adj_tile2d<POL, M, P, HJB>(g, c, a, s);
         const int width = 2 * NT - 2 * Gm::HC - 2;
         const int strips = (g.nx + width - 1) / width;
         static int sms = -1;
@@ -466,8 +474,9 @@ struct AdjLauncher {
 // TE writes jbar_x, jbar_y when either is asked for; TM writes jbar_z when asked
 template <int M, int P>
 int adj_pair(const Geo &g, const Coef2 &c, const Adj2dArgs<float> &a, cudaStream_t s) {
-    if (a.Jbo[0] || a.Jbo[1]) AdjLauncher<TE, M, P, true>::run(g, c, a, s);
-    else AdjLauncher<TE, M, P, false>::run(g, c, a, s);
+    const cudaStream_t te = t_adj_te ? t_adj_te : s;
+    if (a.Jbo[0] || a.Jbo[1]) AdjLauncher<TE, M, P, true>::run(g, c, a, te);
+    else AdjLauncher<TE, M, P, false>::run(g, c, a, te);
     if (a.Jbo[2]) AdjLauncher<TM, M, P, true>::run(g, c, a, s);
     else AdjLauncher<TM, M, P, false>::run(g, c, a, s);
     return 2;
@@ -486,17 +495,25 @@ int adj_p(const Geo &g, const Coef2 &c, const Adj2dArgs<float> &a, cudaStream_t 
 
 }  // namespace
 
-bool adjoint2d_supported(const Geo &g, int m, int passes) {
-    return g.nz == 1 && g.nx % 2 == 0 && (int64_t)g.ny * g.pitch < ((int64_t)1 << 31) && m >= 0 && m <= 4 &&
+bool adjoint2d_supported(const Geo &g, int m, int passes, int seg_rows) {
+    // odd n_x: on register tiles only (the row pipeline loads column pairs)
+    return g.nz == 1 && (g.nx % 2 == 0 || (seg_rows == 0 && fused2d_tiles(g))) && (int64_t)g.ny * g.pitch < ((int64_t)1 << 31) && m >= 0 && m <= 4 &&
            passes >= 0 && passes <= 3;
 }
 
-int launch_adjoint2d(const Geo &g, const Coef<float> &c, const Adj2dArgs<float> &a, cudaStream_t s, int seg_rows) {
-    if (!adjoint2d_supported(g, a.m, a.passes) || c.c6 != 1.f / 6.f) return -1;
-    struct RowsScope {  // the segment rows of this call's launches
-        explicit RowsScope(int r) { t_adj_rows = r; }
-        ~RowsScope() { t_adj_rows = 0; }
-    } rows_scope(seg_rows);
+int launch_adjoint2d(const Geo &g, const Coef<float> &c, const Adj2dArgs<float> &a, cudaStream_t s, int seg_rows,
+                     cudaStream_t s_te) {
+    if (!adjoint2d_supported(g, a.m, a.passes, seg_rows) || c.c6 != 1.f / 6.f) return -1;
+    struct RowsScope {  // the segment rows and the TE stream of this call's launches
+        RowsScope(int r, cudaStream_t te) {
+            t_adj_rows = r;
+            t_adj_te = te;
+        }
+        ~RowsScope() {
+            t_adj_rows = 0;
+            t_adj_te = nullptr;
+        }
+    } rows_scope(seg_rows, s_te);
     Coef2 k;
     auto b = [](float v) { return make_float2(v, v); };
     k.kx = b(c.kx);

@@ -19,13 +19,12 @@
 
 #include "fused2d.h"
 #include "pol_tile.cuh"
+#include "tile2d.cuh"
 
 namespace fmx {
 namespace {
 
-using namespace pair2;
-
-constexpr unsigned FULL = 0xffffffffu;
+using namespace tile2d;
 
 // Grids of at most this many cells run both sets in one launch on the grid's
 // own stream: their tiles (48 x 49 columns and rows, both sets) leave SMs free
@@ -39,34 +38,7 @@ struct TileHalo {
     static constexpr int HC = (M + PX + 1) / 2 * 2;  // columns left of the tile (even) and right of it
 };
 
-__device__ __forceinline__ float up1(float v) { return __shfl_up_sync(FULL, v, 1); }
-__device__ __forceinline__ float dn1(float v) { return __shfl_down_sync(FULL, v, 1); }
-__device__ __forceinline__ f2 sub(f2 a, f2 b) { return fma(b, m1(), a); }
-// columns 2t-1 and 2t+2 beside the own pair: f[i-1] + f[i+1]
-__device__ __forceinline__ f2 xsum(f2 v, float l, float r) { return mk(l + v.y, v.x + r); }
-
-// unnormalised (2P+1)-tap binomial along x of a warp's columns, the taps
-// folded in the order of binom_taps
-template <int P>
-__device__ __forceinline__ f2 binom_x(f2 v) {
-    float col[2 * P + 2];  // columns 2t-P .. 2t+1+P
-#pragma unroll
-    for (int i = 0; i < 2 * P + 2; ++i) {
-        const int off = i - P, pr = off >= 0 ? off / 2 : -((1 - off) / 2);  // pair t + pr
-        const float w = (off - 2 * pr) ? v.y : v.x;
-        col[i] = pr == 0 ? w : (pr < 0 ? __shfl_up_sync(FULL, w, -pr) : __shfl_down_sync(FULL, w, pr));
-    }
-    f2 acc = mk(col[0] + col[2 * P], col[1] + col[2 * P + 1]);
-#pragma unroll
-    for (int k = 1; k < P; ++k) acc = fma(cst(binom2(P, k)), mk(col[k] + col[2 * P - k], col[k + 1] + col[2 * P + 1 - k]), acc);
-    return fma(cst(binom2(P, P)), v, acc);
-}
-
-struct Tile2dGeo {
-    int tw, th, ntx, nty;  // columns and rows a tile writes, tiles along x and y
-};
-
-template <int POL, int M, int P, bool HJ, int R, int NW, bool SEAM>
+template <int POL, int M, int P, bool HJ, bool SEAM>
 __device__ __forceinline__ void tile_step(const Fused2dArgs<float> &a, const Geo &g, const Coef2 &c, int tw, int th,
                                           int x0, int y0, float2 *sm) {
     using H = TileHalo<M, P, HJ>;
@@ -205,66 +177,8 @@ __device__ __forceinline__ void tile_step(const Fused2dArgs<float> &a, const Geo
         }
     }
     // ---------------- sweeps ----------------
-    auto publish = [&](int buf) {
-        pub(buf, 0, wp) = d[0][R - 1];
-        pub(buf, 1, wp) = d[0][0];
-        if constexpr (POL == TE) pub(buf, 2, wp) = d[1][R - 1];
-    };
+    sweeps<POL, M>(d, c, wp, wb, wa, row, pub, [&](int s) { return need(s - M, th + M - s); });
     f2 e[NC][R], bf[NB][R];  // E^n of the own rows; B again for the Faraday update
-#pragma unroll
-    for (int s = 1; s <= M; ++s) {
-        const int buf = (s - 1) & 1;
-        publish(buf);
-        __syncthreads();
-        if (s == 1) {
-            // the raw current is consumed: its rows now keep dE' (own rows only)
-#pragma unroll
-            for (int q = 0; q < NC; ++q)
-#pragma unroll
-                for (int j = 0; j < R; ++j) row(q, wp * R + j) = d[q][j];
-        }
-        if (!need(s - M, th + M - s)) continue;
-        if constexpr (POL == TE) {
-            // h = Dbar_x Ex, gy = Dbar_y Ey
-            auto dx = [&](f2 v) { return mk(v.x - up1(v.y), v.y - v.x); };
-            f2 xp = pub(buf, 0, wb), yp = pub(buf, 2, wb), h = dx(d[0][0]);
-            const f2 xa = pub(buf, 1, wa);
-            float eyrp = dn1(yp.x);
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                const f2 x = d[0][j], y = d[1][j], xn = j < R - 1 ? d[0][j + 1] : xa;
-                const f2 dp0 = s == 1 ? x : row(0, wp * R + j), dp1 = s == 1 ? y : row(1, wp * R + j);
-                const float eyl = up1(y.y), eyr = dn1(y.x);
-                const f2 gy = sub(y, yp), hn = dx(xn);
-                f2 o0 = fma(c.ay, fma(x, m2(), add(xn, xp)), dp0);
-                o0 = fma(c.bxy, mk(gy.y - gy.x, (eyr - eyrp) - gy.y), o0);
-                f2 o1 = fma(c.ax, fma(y, m2(), xsum(y, eyl, eyr)), dp1);
-                o1 = fma(c.bxy, sub(hn, h), o1);
-                d[0][j] = o0;
-                d[1][j] = o1;
-                xp = x;
-                yp = y;
-                h = hn;
-                eyrp = eyr;
-            }
-        } else {
-            auto dxx = [&](f2 v) { return fma(v, m2(), xsum(v, up1(v.y), dn1(v.x))); };
-            f2 zp = pub(buf, 0, wb), Dp = dxx(zp), D = dxx(d[0][0]);
-            const f2 za = pub(buf, 1, wa);
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                const f2 z = d[0][j], zn = j < R - 1 ? d[0][j + 1] : za;
-                const f2 dp0 = s == 1 ? z : row(0, wp * R + j);
-                const f2 Dn = dxx(zn);
-                f2 o0 = fma(c.ax, D, dp0);
-                o0 = fma(c.ay, fma(z, m2(), add(zn, zp)), o0);
-                d[0][j] = fma(c.axy, fma(D, m2(), add(Dn, Dp)), o0);
-                zp = z;
-                Dp = D;
-                D = Dn;
-            }
-        }
-    }
     // ---------------- E and Faraday updates ----------------
     const bool act = need(0, th);
     {
@@ -324,7 +238,6 @@ __device__ __forceinline__ void tile_step(const Fused2dArgs<float> &a, const Geo
 
 // SET: the TE or the TM set, or BOTH (blockIdx.y picks it)
 constexpr int BOTH = 2;
-constexpr int R = 8, NW = 8;
 
 template <int SET, int M, int P, bool HJ>
 __global__ void __launch_bounds__(32 * NW, 2) k_tile2d(Fused2dArgs<float> a, Geo g, Coef2 c, Tile2dGeo t) {
@@ -339,30 +252,13 @@ __global__ void __launch_bounds__(32 * NW, 2) k_tile2d(Fused2dArgs<float> a, Geo
     const bool seam = (g.nx & 1) && (x0 < HC || x0 - HC + 64 > g.nx);
     const bool tm = SET == TM || (SET == BOTH && blockIdx.y == 1);
     if (SET != TM && !tm) {
-        if (!seam) tile_step<TE, M, P, HJ, R, NW, false>(a, g, c, t.tw, th, x0, y0, tsm);
-        else tile_step<TE, M, P, HJ, R, NW, true>(a, g, c, t.tw, th, x0, y0, tsm);
+        if (!seam) tile_step<TE, M, P, HJ, false>(a, g, c, t.tw, th, x0, y0, tsm);
+        else tile_step<TE, M, P, HJ, true>(a, g, c, t.tw, th, x0, y0, tsm);
     }
     if (SET != TE && tm) {
-        if (!seam) tile_step<TM, M, P, HJ, R, NW, false>(a, g, c, t.tw, th, x0, y0, tsm);
-        else tile_step<TM, M, P, HJ, R, NW, true>(a, g, c, t.tw, th, x0, y0, tsm);
+        if (!seam) tile_step<TM, M, P, HJ, false>(a, g, c, t.tw, th, x0, y0, tsm);
+        else tile_step<TM, M, P, HJ, true>(a, g, c, t.tw, th, x0, y0, tsm);
     }
-}
-
-// tiles of equal size that cover the grid, none larger than the halo leaves
-// of 64 columns and R NW rows
-template <int M, int P, bool HJ>
-Tile2dGeo tile_geo(const Geo &g) {
-    using H = TileHalo<M, P, HJ>;
-    constexpr int TWX = (63 - H::HC - M - H::PX) / 2 * 2, THX = R * NW - 2 * H::HY - 1;
-    static_assert(TWX >= 2 && THX >= 1 && R >= P, "halo larger than the tile");
-    Tile2dGeo t;
-    t.ntx = (g.nx + TWX - 1) / TWX;
-    t.tw = ((g.nx + t.ntx - 1) / t.ntx + 1) / 2 * 2;
-    t.ntx = (g.nx + t.tw - 1) / t.tw;
-    t.nty = (g.ny + THX - 1) / THX;
-    t.th = (g.ny + t.nty - 1) / t.nty;
-    t.nty = (g.ny + t.th - 1) / t.th;
-    return t;
 }
 
 }  // namespace
@@ -374,7 +270,11 @@ void launch_tile2d(const Geo &g, const Coef2 &c, const Fused2dArgs<float> &a, cu
     static const bool attr =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
     (void)attr;  // a failure shows up in the launch
-    const Tile2dGeo t = tile_geo<M, P, HJ>(g);
+    // what the halo leaves of 64 columns and R NW rows
+    using H = TileHalo<M, P, HJ>;
+    constexpr int TWX = (63 - H::HC - M - H::PX) / 2 * 2, THX = R * NW - 2 * H::HY - 1;
+    static_assert(TWX >= 2 && THX >= 1 && R >= P, "halo larger than the tile");
+    const Tile2dGeo t = cover(g.nx, g.ny, TWX, THX);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(t.ntx * t.nty, SET == BOTH ? 2 : 1);
     cfg.blockDim = dim3(32 * NW);
