@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(CNT) k3_source1(Geo g, Coef<T> c, const T *b0,
 // walks the planes of its column, E of the plane above carried over; the
 // neighbours x+1 and y+1 come through L1.  Bound by memory; the
 // one-thread-per-cell kernel spent its time on periodic 64-bit indices (201 x
-// 150 x 99 FP32 26.5 -> 20.5 us).
+// 150 x 99 FP32 26.5 -> 20.5 us, 128 x 128 x 96 FP64 49 -> 42).
 template <typename T>
 __global__ void __launch_bounds__(256) k3_faraday1(Geo g, Coef<T> c, const T *__restrict__ e0, const T *__restrict__ e1,
                                                    const T *__restrict__ e2, T *__restrict__ b0, T *__restrict__ b1,
@@ -528,7 +528,10 @@ __device__ __forceinline__ PlaneTerms plane_terms(const F &V, const Coef3P &c, f
 // (nothing else of the plane is read again), adds its terms to the partial
 // outputs held in registers, and completes output plane z0+i-2.  One plane
 // is read while the next RS-1 are on their way; one barrier per plane.
-template <bool UPD>
+// FIRST: the first sweep, whose input is dE' itself: the own pair of an output
+// plane was read from the ring one iteration before, so dE' is not fetched a
+// second time (512^3: 822 -> 689 us).
+template <bool UPD, bool FIRST>
 __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, const float *p0, const float *p1,
                                                              const float *p2, const float *i0, const float *i1,
                                                              const float *i2, float *o0, float *o1, float *o2, int zseg) {
@@ -566,14 +569,19 @@ __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, c
             pd[b][q] = mk(0.f, 0.f);
             pe[b][q] = mk(0.f, 0.f);
             if (ok) {
-                pd[b][q] = __ldg(reinterpret_cast<const float2 *>(dp[q] + pcell));
+                if (!FIRST) pd[b][q] = __ldg(reinterpret_cast<const float2 *>(dp[q] + pcell));
                 if (UPD) pe[b][q] = *reinterpret_cast<const float2 *>(out[q] + pcell);
             }
         }
         pcell += g.plane;
     };
-    prefetch(0, inside);
-    prefetch(1, inside && z0 + 1 < z1);
+    if (!FIRST || UPD) {
+        prefetch(0, inside);
+        prefetch(1, inside && z0 + 1 < z1);
+    }
+    f2 pv[3];  // FIRST: the own pair of the plane before
+#pragma unroll
+    for (int q = 0; q < 3; ++q) pv[q] = mk(0.f, 0.f);
     const f2 bxy6 = mul(c.bxy, c.c6);
     f2 xa = mk(0.f, 0.f), xb = xa, ya = xa, yb = xa, za = xa;  // partial outputs o, o+1
     auto step = [&](int i, auto bsel) {
@@ -594,12 +602,16 @@ __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, c
                 f2 r[3] = {add(xa, t.x1), add(ya, t.y1), add(za, t.zh)};
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    r[q] = add(pd[b][q], r[q]);
+                    r[q] = add(FIRST ? pv[q] : pd[b][q], r[q]);
                     if (UPD) r[q] = add(pe[b][q], r[q]);
                     *reinterpret_cast<float2 *>(out[q] + ocell) = r[q];
                 }
                 ocell += g.plane;
-                prefetch(b, z0 + i < z1);  // output z0 + i, two iterations on
+                if (!FIRST || UPD) prefetch(b, z0 + i < z1);  // output z0 + i, two iterations on
+            }
+            if (FIRST) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) pv[q] = V(q, 0, 0);
             }
             xa = add(xb, t.x0);
             xb = t.xl;
@@ -622,11 +634,15 @@ __global__ void __launch_bounds__(NTH, UPD ? 2 : 3) k3_sweep2(Geo g, Coef3P c, c
 //   x: k_y (V_k + c6 Dzz V) - k_z (U_k - U_(k-1)),    V = Dbar_y(bwd) Bz,  U = By + c6 Dbar_yy By,
 //   y: k_z (W_k - W_(k-1)) - k_x (V'_k + c6 Dzz V'),  V' = Dbar_x(bwd) Bz, W = Bx + c6 Dbar_xx Bx,
 //   z: k_x Dbar_x(bwd) U - k_y Dbar_y(bwd) W          (in-plane),
-// so plane j of B reaches outputs j-1, j, j+1 through terms of plane j alone.
+// so plane j of B reaches outputs j-1, j, j+1 through terms of plane j, and U and
+// W of plane j-1 (their z-differences are taken before the factor: on smooth
+// fields a difference is exact where the products' sum would round at |B|; with
+// it the source spills nothing and 512^3 takes 5.39 ms a step against 5.50).
 struct CurlTerms {
-    f2 x1, x0, xl;  // x: to outputs j-1 and j+1 (x1), to j (x0), to j+1 (xl = x1 + k_z U)
-    f2 y1, y0, yl;  // y: the same with V' and W
-    f2 z;           // z: to output j
+    f2 x1, x0;  // x: to outputs j-1 and j+1 (x1), to j (x0, without k_z (U - U_(j-1)))
+    f2 y1, y0;  // y: the same with V', and W
+    f2 U, W;
+    f2 z;       // z: to output j
 };
 
 template <typename F>
@@ -645,14 +661,13 @@ __device__ __forceinline__ CurlTerms curl_plane_terms(const F &V, const Coef3P &
     const f2 U = fma(c.c6, d2(by_p, by_0, by_m), by_0), Ul = fma(c.c6, d2(byl_p, byl_0, byl_m), byl_0);
     const f2 W = fma(c.c6, d2(bxr_0, bx_0, bxl_0), bx_0), Wm = fma(c.c6, d2(bxr_m, bx_m, bxl_m), bx_m);
     const f2 Vy = sub(bz_0, bz_m), Vx = sub(bz_0, bzl_0);
-    const f2 kzU = mul(c.kz, U), kzW = mul(c.kz, W);
     CurlTerms t;
     t.x1 = mul(kyc6, Vy);
-    t.x0 = fma(t.x1, m2(), sub(mul(c.ky, Vy), kzU));
-    t.xl = add(t.x1, kzU);
+    t.x0 = fma(t.x1, m2(), mul(c.ky, Vy));
     t.y1 = mul(nkxc6, Vx);
-    t.y0 = fma(t.y1, m2(), sub(kzW, mul(c.kx, Vx)));
-    t.yl = sub(t.y1, kzW);
+    t.y0 = fma(t.y1, m2(), mul(mul(c.kx, Vx), m1()));
+    t.U = U;
+    t.W = W;
     t.z = sub(mul(c.kx, sub(U, Ul)), mul(c.ky, sub(W, Wm)));
     return t;
 }
@@ -691,6 +706,7 @@ __global__ void __launch_bounds__(NTH, 3) k3_source2(Geo g, Coef3P c, const floa
     int64_t ocell = (int64_t)z0 * g.plane + (int64_t)py * g.pitch + px;
     const f2 nkxc6 = mul(mul(c.kx, c.c6), m1()), kyc6 = mul(c.ky, c.c6);
     f2 xa = mk(0.f, 0.f), xb = xa, ya = xa, yb = xa, za = xa;  // partial outputs o, o+1
+    f2 up = xa, wp = xa;  // U and W of the plane before
     // PASSES = 1: x-y binomial of the current of planes j-2, j-1 (own pair);
     // PASSES = 0: the raw current of plane j-1 in jz[a][1]
     f2 jz[3][2];
@@ -745,10 +761,12 @@ __global__ void __launch_bounds__(NTH, 3) k3_source2(Geo g, Coef3P c, const floa
                 for (int q = 0; q < 3; ++q) *reinterpret_cast<float2 *>(out[q] + ocell) = d[q];
                 ocell += g.plane;
             }
-            xa = add(xb, t.x0);
-            xb = t.xl;
-            ya = add(yb, t.y0);
-            yb = t.yl;
+            xa = fma(mul(c.kz, fma(up, m1(), t.U)), m1(), add(xb, t.x0));
+            xb = t.x1;
+            ya = fma(c.kz, fma(wp, m1(), t.W), add(yb, t.y0));
+            yb = t.y1;
+            up = t.U;
+            wp = t.W;
             za = t.z;
             if constexpr (HJ) {
 #pragma unroll
@@ -1063,15 +1081,15 @@ void run_source2(const Geo &g, const Coef<float> &c, const float *const B[3], co
 }
 bool pair_path(const Geo &, double *) { return false; }
 
-template <bool UPD>
+template <bool UPD, bool FIRST>
 void run_sweep2(const Geo &g, const Coef<float> &c, const float *const dEp[3], const float *const in[3],
                 float *const out[3], cudaStream_t s) {
     constexpr size_t bytes = (size_t)SWEEP_RS * 3 * PL2 * sizeof(float);
-    static const int res = resident(k3_sweep2<UPD>, NTH, bytes);
+    static const int res = resident(k3_sweep2<UPD, FIRST>, NTH, bytes);
     const Coef3P cp = coef3p(c);
     int zseg;
     const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
-    k3_sweep2<UPD><<<grid, dim3(TXP, TY), bytes, s>>>(g, cp, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0],
+    k3_sweep2<UPD, FIRST><<<grid, dim3(TXP, TY), bytes, s>>>(g, cp, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0],
                                                      out[1], out[2], zseg);
 }
 
@@ -1139,8 +1157,9 @@ int launch_march3d_sweep(const Geo &g, const Coef<T> &c, const T *const dEp[3], 
                          cudaStream_t s, bool update) {
     if constexpr (std::is_same<T, float>::value) {
         if (pair_path(g, (float *)nullptr)) {
-            if (update) run_sweep2<true>(g, c, dEp, in, out, s);
-            else run_sweep2<false>(g, c, dEp, in, out, s);
+            const bool first = in[0] == dEp[0] && in[1] == dEp[1] && in[2] == dEp[2];
+            if (update) first ? run_sweep2<true, true>(g, c, dEp, in, out, s) : run_sweep2<true, false>(g, c, dEp, in, out, s);
+            else first ? run_sweep2<false, true>(g, c, dEp, in, out, s) : run_sweep2<false, false>(g, c, dEp, in, out, s);
             return 1;
         }
     }
