@@ -34,7 +34,7 @@ template <int POL, int M, int P, bool HJ, int NT, bool L1PF>
 __global__ void __launch_bounds__(NT, 3)
     k_pol2d(Fused2dArgs<float> a, Geo g, Coef2 c, int W, int L, int nstrip) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    pol_tile<POL, M, P, HJ, NT, false, false, L1PF>(a, g, c, W, L, blockIdx.x % nstrip, blockIdx.x / nstrip,
+    pol_tile<POL, M, P, HJ, NT, false, false, L1PF, false>(a, g, c, W, L, blockIdx.x % nstrip, blockIdx.x / nstrip,
                                                     reinterpret_cast<float *>(smraw));
 }
 

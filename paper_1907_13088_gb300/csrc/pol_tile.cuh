@@ -90,8 +90,13 @@ struct PolSmem {
 // synchronises on its own named barrier 1 + half, so that a CTA can carry
 // two independent narrow tiles; otherwise the whole CTA runs it.  L1PF: the
 // input rows are also prefetched into L1 PolPrefetch::L1 rows beyond the
-// register loads (for grids whose rows come from HBM).
-template <int POL, int M, int P, bool HJ, int NT, bool SEAM = false, bool HALF = false, bool L1PF = false>
+// register loads (for grids whose rows come from HBM).  ALIGN: the segment
+// starts at a row that is a multiple of 4 (two to five rows early; the batched
+// kernel, whose four tile bodies share one register budget, compiles worse
+// without: 531 -> 573 us at its best choice; the single-grid kernel is 1.9%
+// faster without, 4096^2 241 -> 236.5 us per step).
+template <int POL, int M, int P, bool HJ, int NT, bool SEAM = false, bool HALF = false, bool L1PF = false,
+          bool ALIGN = true>
 __device__ __forceinline__ void pol_tile(const Fused2dArgs<float> &a, const Geo &g, const Coef2 &c, int W, int L,
                                          int strip, int seg, float *sm, int half = 0) {
     using G = PolGeom<M, P, HJ>;
@@ -156,9 +161,11 @@ __device__ __forceinline__ void pol_tile(const Fused2dArgs<float> &a, const Geo 
     float *__restrict__ oB0 = POL == TE ? a.Bo[2] : a.Bo[0];
     float *__restrict__ oB1 = a.Bo[1];
 
-    // first row, aligned down to a multiple of 4 (extra warm-up rows are harmless)
-    int r0 = y0 - M - G::WU - 1;
-    r0 -= ((r0 % 4) + 4) % 4;
+    // first row: the earliest that a window reaches (ring slots and unroll go by
+    // a row's distance from it), or aligned down to a multiple of 4 (extra
+    // warm-up rows are harmless)
+    int r0 = y0 - M - G::WU - (ALIGN ? 1 : 0);
+    if (ALIGN) r0 -= ((r0 % 4) + 4) % 4;
     int r1 = y1 + 2 * M + 1;
     r1 += (4 - ((r1 - r0) % 4)) % 4;
 
@@ -266,7 +273,7 @@ __device__ __forceinline__ void pol_tile(const Fused2dArgs<float> &a, const Geo 
 #pragma unroll
         for (int k = 0; k < PE; ++k) pe1[k] = z2;
     }
-    int b0 = ((r0 % D0) + D0) % D0;  // dE' ring slot of row r0 (a multiple of 4)
+    int b0 = ALIGN ? ((r0 % D0) + D0) % D0 : 0;  // dE' ring slot of row r0 (a multiple of 4)
     // With D0 = 12 the dE' ring is addressed through the bases of its three
     // 4-row groups, rotated once per block of four rows, so that every slot a
     // row touches is a compile-time offset from one of them (no per-access
