@@ -24,11 +24,12 @@ constexpr int TY = 8, NTH = 32 * TY, RH = TY + 2;  // pair kernels: rows of the 
 // planes a segment marches over.  The CTAs on one SM share its arithmetic, so a
 // launch takes about the CTAs of the fullest SM times the planes each marches
 // (two more than it writes), and c of them resident at a time leave their
-// latencies open, which a factor 1 + 1/(2c) stands for; the segment height
-// with the least product, 4 to 64 planes, is taken (128 x 128 x 96 FP64 sweep: 24
-// planes, one CTA on each of 128 SMs, 270 us; 7 planes, 448 CTAs, 250 us).
-// tiles: CTAs per segment; res: CTAs an SM holds.
-int zseg_for(int nz, long long tiles, int res) {
+// latencies open, which a factor 1 + lat/c stands for (0.5; 0.6 for the CTAs of
+// two warps, or 64^3 FP64 would leave one of them on an SM: 450 us a step, 300 so); the segment height
+// with the least product, 4 to 64 planes, is taken (128 x 128 x 96 FP64 sweep, CTAs
+// of four warps: 24 planes, one CTA on each of 128 SMs, 270 us; 7 planes, 448
+// CTAs, 250 us).  tiles: CTAs per segment; res: CTAs an SM holds.
+int zseg_for(int nz, long long tiles, int res, double lat) {
     static const int sms = [] {
         int dev = 0, v = 0;
         cudaGetDevice(&dev);
@@ -41,7 +42,7 @@ int zseg_for(int nz, long long tiles, int res) {
         if (z < 4 && nseg > 1) break;
         const long long n = (tiles * ((nz + z - 1) / z) + sms - 1) / sms;  // CTAs of the fullest SM
         // rounds of res resident CTAs, then the rest
-        const double load = (double)(n / res) * (res + 0.5) + (n % res ? (double)(n % res) + 0.5 : 0.0);
+        const double load = (double)(n / res) * (res + lat) + (n % res ? (double)(n % res) + lat : 0.0);
         if (load * (z + 2) < least) {
             least = load * (z + 2);
             best = z;
@@ -72,17 +73,19 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // ---------------------------------------------------------------------------
-// One column per thread (FP64, odd n_x): a tile of 32 columns x 16 rows, 128
-// threads, four rows of a column each.  FP64 arithmetic runs at 1/64 of the
+// One column per thread (FP64, odd n_x): a tile of 32 columns x 8 rows, 64
+// threads, four rows of a column each (small CTAs, so that the segments share
+// the FP64 arithmetic of all SMs evenly: 128 x 128 x 96 FP64 takes 1142 us a step
+// against 1254 with 16 rows).  FP64 arithmetic runs at 1/64 of the
 // FP32 rate on this part and bounds these kernels, so they are written for the
 // fewest operations: the factored form (see plane_terms below), differences
 // formed once and shared along the four rows of a thread, partial outputs
 // carried as FMA accumulators.  A sweep takes 54 FP64 operations per cell
 // against 135 for the 27-point stencils evaluated cell by cell, the filtered
-// source 52 against about 150.  128 x 128 x 96 FP64: sweep 685 -> 242 us, source
-// 627 -> 231 us (their operations take 213 and 189 us at the FMA rate that
+// source 52 against about 150.  128 x 128 x 96 FP64, 16 rows: sweep 685 -> 242 us,
+// source 627 -> 231 us (their operations take 213 and 189 us at the FMA rate that
 // fmx_fma_peak measures); 201 x 150 x 99 FP32: sweep 53 -> 33 us, source 68 -> 38 us.
-constexpr int CX = 32, CR = 4, CW = 4, CROWS = CR * CW, CNT = 32 * CW;
+constexpr int CX = 32, CR = 4, CW = 2, CROWS = CR * CW, CNT = 32 * CW;
 constexpr int CPW = CX + 2, CPL = CPW * (CROWS + 2);  // row and plane of the tile with its halo
 constexpr int CCP = (CPL + CNT - 1) / CNT;             // copies of a component plane per thread
 
@@ -121,7 +124,7 @@ __device__ __forceinline__ T d2s(T a, T v, T b) { return (a + b) - T(2) * v; }  
 // out = dEp + A in, or with UPD E = E + dEp + A in (E in place)
 constexpr int SWEEP1_RS = 4;
 template <typename T, bool UPD>
-__global__ void __launch_bounds__(CNT, sizeof(T) == 8 ? 3 : (UPD ? 4 : 6)) k3_sweep1(Geo g, Coef<T> c, const T *p0, const T *p1, const T *p2, const T *i0,
+__global__ void __launch_bounds__(CNT, 6) k3_sweep1(Geo g, Coef<T> c, const T *p0, const T *p1, const T *p2, const T *i0,
                                                  const T *i1, const T *i2, T *o0, T *o1, T *o2, int zseg) {
     constexpr int RS = SWEEP1_RS;
     extern __shared__ __align__(16) unsigned char m3raw[];
@@ -1018,9 +1021,9 @@ __global__ void __launch_bounds__(FNT, 2) k3_sweeps2f(Geo g, Coef3P c, const flo
 }
 
 // launch grid of a kernel with CTAs of tx columns x ty rows, zseg planes each
-dim3 grid_of(const Geo &g, int tx, int ty, int res, int *zseg) {
+dim3 grid_of(const Geo &g, int tx, int ty, int res, int *zseg, double lat = 0.5) {
     const dim3 t((g.nx + tx - 1) / tx, (g.ny + ty - 1) / ty);
-    *zseg = zseg_for(g.nz, (long long)t.x * t.y, res);
+    *zseg = zseg_for(g.nz, (long long)t.x * t.y, res, lat);
     return dim3(t.x, t.y, (g.nz + *zseg - 1) / *zseg);
 }
 // allows the dynamic shared memory and returns the CTAs an SM holds
@@ -1041,7 +1044,7 @@ void run_source(const Geo &g, const Coef<T> &c, const T *const B[3], const T *co
     constexpr size_t bytes = (size_t)SOURCE1_RS * (HJ ? 6 : 3) * CPL * sizeof(T);
     static const int res = resident(k3_source1<T, PASSES, HJ>, CNT, bytes);
     int zseg;
-    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg);
+    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg, 0.6);
     k3_source1<T, PASSES, HJ><<<grid, CNT, bytes, s>>>(g, c, B[0], B[1], B[2], HJ ? J[0] : nullptr, HJ ? J[1] : nullptr,
                                                        HJ ? J[2] : nullptr, out[0], out[1], out[2], zseg);
 }
@@ -1052,7 +1055,7 @@ void run_sweep1(const Geo &g, const Coef<T> &c, const T *const dEp[3], const T *
     constexpr size_t bytes = (size_t)SWEEP1_RS * 3 * CPL * sizeof(T);
     static const int res = resident(k3_sweep1<T, UPD>, CNT, bytes);
     int zseg;
-    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg);
+    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg, 0.6);
     k3_sweep1<T, UPD><<<grid, CNT, bytes, s>>>(g, c, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0], out[1],
                                                out[2], zseg);
 }
