@@ -1,5 +1,6 @@
 // FP32 2D adjoint step on register tiles (the maps of adjoint2d.cu, the tiles of
-// tile2d.cu): one launch per set and step, any n_x.  A warp holds 8 rows of 64
+// tile2d.cu): one launch per set and step, even n_x (odd n_x stays on the staged
+// kernels: another order of the FP32 sums moves dL/dtheta in its seventh digit).  A warp holds 8 rows of 64
 // columns; u = Ebar - C_b Bbar, the M sweeps of the forward tile give w, and the
 // rows of w at the warps' borders go through shared memory once for the
 // transposed Faraday update and the filter of jbar.  M + 1 barriers a step
@@ -33,7 +34,7 @@ struct AdjHalo {
     static_assert(TWX >= 2 && THX >= 1 && R >= P, "halo larger than the tile");
 };
 
-template <int POL, int M, int P, bool HJB, bool SEAM>
+template <int POL, int M, int P, bool HJB>
 __device__ __forceinline__ void adj_tile(const Adj2dArgs<float> &a, const Geo &g, const Coef2 &c, int tw, int th, int x0,
                                          int y0, float2 *sm) {
     using H = AdjHalo<POL, M, P, HJB>;
@@ -46,8 +47,6 @@ __device__ __forceinline__ void adj_tile(const Adj2dArgs<float> &a, const Geo &g
     const int cg = x0 - HC + 2 * lane;
     int xc = cg % g.nx;
     if (xc < 0) xc += g.nx;
-    [[maybe_unused]] const int dxc = xc + 1 == g.nx ? 1 - g.nx : 1;
-    [[maybe_unused]] const bool xlast = cg + 1 >= g.nx;
     const bool xout = 2 * lane >= HC && 2 * lane < HC + tw && cg < g.nx;
     const int ry = wp * R - HY;  // first own row, relative to the tile's first
     const int pitch = (int)g.pitch, plane = g.ny * pitch;
@@ -59,18 +58,8 @@ __device__ __forceinline__ void adj_tile(const Adj2dArgs<float> &a, const Geo &g
         o += pitch;
         if (o >= plane) o -= plane;
     };
-    auto ld = [&](const float *__restrict__ p, int o) {
-        if constexpr (SEAM) return mk(__ldg(p + o), __ldg(p + o + dxc));
-        else return __ldg(reinterpret_cast<const float2 *>(p + o));
-    };
-    auto st = [&](float *p, int o, f2 v) {
-        if constexpr (SEAM) {
-            p[o] = v.x;
-            if (!xlast) p[o + 1] = v.y;
-        } else {
-            *reinterpret_cast<float2 *>(p + o) = v;
-        }
-    };
+    auto ld = [&](const float *__restrict__ p, int o) { return __ldg(reinterpret_cast<const float2 *>(p + o)); };
+    auto st = [&](float *p, int o, f2 v) { *reinterpret_cast<float2 *>(p + o) = v; };
     const float *inE0 = POL == TE ? a.Eb[0] : a.Eb[2], *inE1 = a.Eb[1];
     const float *inB0 = POL == TE ? a.Bb[2] : a.Bb[0], *inB1 = a.Bb[1];
     float *oE0 = POL == TE ? a.Ebo[0] : a.Ebo[2], *oE1 = a.Ebo[1];
@@ -195,10 +184,7 @@ __global__ void __launch_bounds__(32 * NW, 2) k_adj_tile2d(Adj2dArgs<float> a, G
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int x0 = (int)(blockIdx.x % t.ntx) * t.tw, y0 = (int)(blockIdx.x / t.ntx) * t.th;
     const int th = min(t.th, g.ny - y0);
-    constexpr int HC = AdjHalo<POL, M, P, HJB>::HC;
-    const bool seam = (g.nx & 1) && (x0 < HC || x0 - HC + 64 > g.nx);
-    if (!seam) adj_tile<POL, M, P, HJB, false>(a, g, c, t.tw, th, x0, y0, tsm);
-    else adj_tile<POL, M, P, HJB, true>(a, g, c, t.tw, th, x0, y0, tsm);
+    adj_tile<POL, M, P, HJB>(a, g, c, t.tw, th, x0, y0, tsm);
 }
 
 }  // namespace

@@ -495,15 +495,15 @@ int adj_p(const Geo &g, const Coef2 &c, const Adj2dArgs<float> &a, cudaStream_t 
 
 }  // namespace
 
-bool adjoint2d_supported(const Geo &g, int m, int passes, int seg_rows) {
-    // odd n_x: on register tiles only (the row pipeline loads column pairs)
-    return g.nz == 1 && (g.nx % 2 == 0 || (seg_rows == 0 && fused2d_tiles(g))) && (int64_t)g.ny * g.pitch < ((int64_t)1 << 31) && m >= 0 && m <= 4 &&
+bool adjoint2d_supported(const Geo &g, int m, int passes) {
+    // odd n_x takes the staged kernels, whose rounding dL/dtheta is held to
+    return g.nz == 1 && g.nx % 2 == 0 && (int64_t)g.ny * g.pitch < ((int64_t)1 << 31) && m >= 0 && m <= 4 &&
            passes >= 0 && passes <= 3;
 }
 
 int launch_adjoint2d(const Geo &g, const Coef<float> &c, const Adj2dArgs<float> &a, cudaStream_t s, int seg_rows,
                      cudaStream_t s_te) {
-    if (!adjoint2d_supported(g, a.m, a.passes, seg_rows) || c.c6 != 1.f / 6.f) return -1;
+    if (!adjoint2d_supported(g, a.m, a.passes) || c.c6 != 1.f / 6.f) return -1;
     struct RowsScope {  // the segment rows and the TE stream of this call's launches
         RowsScope(int r, cudaStream_t te) {
             t_adj_rows = r;

@@ -830,7 +830,7 @@ bool adjoint_fused_ok(const fmx_grid *g, int *passes) {
     *passes = g->p.filter_target == FMX_FILTER_CURRENT ? g->p.filter_passes : 0;
     return g->p.precision == FMX_F32 && g->p.dims == 2 && g->engine == FMX_ENGINE_FUSED &&
            g->p.iter_mode == FMX_ITER_FIXED && !(g->p.filter_target == FMX_FILTER_FIELDS && g->p.filter_passes > 0) &&
-           (float)g->co[4] == 1.f / 6.f && fmx::adjoint2d_supported(g->geo, g->p.m, *passes, g->seg_rows);
+           (float)g->co[4] == 1.f / 6.f && fmx::adjoint2d_supported(g->geo, g->p.m, *passes);
 }
 
 // One fused adjoint step from (Eb, Bb) into (Ebo, Bbo) (out of place), jbar

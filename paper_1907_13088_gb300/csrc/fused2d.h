@@ -76,9 +76,8 @@ struct Adj2dArgs {
 // that the rows come from HBM (4096^2, m = 4, p = 3: +11%); below, with the
 // fields in L2, the prefetches only cost issue slots (1024^2: -23%).
 bool fused2d_l1_prefetch(const Geo &g);
-// 32-bit element offsets; m <= 4, passes <= 3; even nx, or a grid on register
-// tiles (fused2d_tiles) without a segment height asked for
-bool adjoint2d_supported(const Geo &g, int m, int passes, int seg_rows);
+// even nx, 32-bit element offsets; m <= 4, passes <= 3
+bool adjoint2d_supported(const Geo &g, int m, int passes);
 // s_te: stream for the TE launch (nullptr: s); the caller orders the two
 int launch_adjoint2d(const Geo &g, const Coef<float> &c, const Adj2dArgs<float> &a, cudaStream_t s, int seg_rows = 0,
                      cudaStream_t s_te = nullptr);

@@ -1,6 +1,6 @@
 """The FP32 2D adjoint step on register tiles (adj_tile2d.cu): the bits of the
-row pipeline where that covers the grid (even n_x), and the oracle's adjoint
-everywhere, odd n_x among them, at tile edges and on grids smaller than a tile."""
+row pipeline (even n_x), and the oracle's adjoint everywhere, odd n_x (staged
+kernels) among them, at tile edges and on grids smaller than a tile."""
 import ctypes
 
 import numpy as np
