@@ -464,7 +464,7 @@ struct Launcher {
             double least = 1e300;
             for (int n = 1; n <= g.ny; ++n) {
                 const int rows = (g.ny + n - 1) / n;
-                if (rows < 8 && n > 1) break;
+                if (n > 1 && (rows < 8 || (long long)sh.strips * n > 64LL * sms)) break;  // finer only adds rows
                 const long long k = ((long long)sh.strips * ((g.ny + rows - 1) / rows) + sms - 1) / sms;
                 const double load = (double)(k / bps) * (bps + 0.5) + (k % bps ? (double)(k % bps) + 0.5 : 0.0);
                 if (load * (rows + 6) < least) {
