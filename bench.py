@@ -592,8 +592,8 @@ def run_3d(args):
 # (halo and warm-up rows included): (DADD + DMUL + 2 x DFMA) thread
 # instructions of one launch over its output cells, from the ncu capture of
 # k_fused2d<double, 4, 3> at 2048^2 (profiles/k_fused2d_f64_2048.md):
-# (562.4 M + 17.4 M + 2 x 463.8 M) / 2048^2 = 359
-FP64_FLOPS_PER_CELL_STEP_2D = 359
+# (540.9 M + 16.1 M + 2 x 295.1 M) / 2048^2 = 274
+FP64_FLOPS_PER_CELL_STEP_2D = 274
 
 
 def run_f64(args):
