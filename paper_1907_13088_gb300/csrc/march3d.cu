@@ -41,7 +41,6 @@ int zseg_for(int nz, long long tiles, int res, double lat) {
         const int z = (nz + nseg - 1) / nseg;
         if (z < 4 && nseg > 1) break;
         const long long n = (tiles * ((nz + z - 1) / z) + sms - 1) / sms;  // CTAs of the fullest SM
-        if (n > 128 && least < 1e300) break;  // finer only adds planes
         // rounds of res resident CTAs, then the rest
         const double load = (double)(n / res) * (res + lat) + (n % res ? (double)(n % res) + lat : 0.0);
         if (load * (z + 2) < least) {
