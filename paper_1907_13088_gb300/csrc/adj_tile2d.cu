@@ -36,7 +36,7 @@ struct AdjHalo {
 
 template <int POL, int M, int P, bool HJB>
 __device__ __forceinline__ void adj_tile(const Adj2dArgs<float> &a, const Geo &g, const Coef2 &c, int tw, int th, int x0,
-                                         int y0, float2 *sm) {
+                                         int y0, int zero, float2 *sm) {
     using H = AdjHalo<POL, M, P, HJB>;
     constexpr int HY = H::HY, HC = H::HC, NC = POL == TE ? 2 : 1;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -52,13 +52,13 @@ __device__ __forceinline__ void adj_tile(const Adj2dArgs<float> &a, const Geo &g
     const int pitch = (int)g.pitch, plane = g.ny * pitch;
     int yw = (y0 + ry) % g.ny;
     if (yw < 0) yw += g.ny;
-    const int orow0 = yw * pitch + xc;
+    const int orow0 = yw * pitch + xc + zero;
     auto need = [&](int lo, int hi) { return ry <= hi && ry + R - 1 >= lo; };
     auto next_row = [&](int &o) {
         o += pitch;
         if (o >= plane) o -= plane;
     };
-    auto ld = [&](const float *__restrict__ p, int o) { return __ldg(reinterpret_cast<const float2 *>(p + o)); };
+    auto ld = [&](const float *p, int o) { return ld2(p + o); };
     auto st = [&](float *p, int o, f2 v) { *reinterpret_cast<float2 *>(p + o) = v; };
     const float *inE0 = POL == TE ? a.Eb[0] : a.Eb[2], *inE1 = a.Eb[1];
     const float *inB0 = POL == TE ? a.Bb[2] : a.Bb[0], *inB1 = a.Bb[1];
@@ -179,12 +179,10 @@ __device__ __forceinline__ void adj_tile(const Adj2dArgs<float> &a, const Geo &g
 template <int POL, int M, int P, bool HJB>
 __global__ void __launch_bounds__(32 * NW, 2) k_adj_tile2d(Adj2dArgs<float> a, Geo g, Coef2 c, Tile2dGeo t) {
     extern __shared__ __align__(16) float2 tsm[];
-    // nothing is read or written before the kernel before it in the stream is done
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int zero = dependency_wait();
     const int x0 = (int)(blockIdx.x % t.ntx) * t.tw, y0 = (int)(blockIdx.x / t.ntx) * t.th;
     const int th = min(t.th, g.ny - y0);
-    adj_tile<POL, M, P, HJB>(a, g, c, t.tw, th, x0, y0, tsm);
+    adj_tile<POL, M, P, HJB>(a, g, c, t.tw, th, x0, y0, zero, tsm);
 }
 
 }  // namespace

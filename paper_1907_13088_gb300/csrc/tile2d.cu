@@ -40,7 +40,7 @@ struct TileHalo {
 
 template <int POL, int M, int P, bool HJ, bool SEAM>
 __device__ __forceinline__ void tile_step(const Fused2dArgs<float> &a, const Geo &g, const Coef2 &c, int tw, int th,
-                                          int x0, int y0, float2 *sm) {
+                                          int x0, int y0, int zero, float2 *sm) {
     using H = TileHalo<M, P, HJ>;
     constexpr int HY = H::HY, HC = H::HC, NC = POL == TE ? 2 : 1, NB = POL == TE ? 1 : 2;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -65,12 +65,12 @@ __device__ __forceinline__ void tile_step(const Fused2dArgs<float> &a, const Geo
     const int pitch = (int)g.pitch, plane = g.ny * pitch;
     int yw = (y0 + ry) % g.ny;
     if (yw < 0) yw += g.ny;
-    const int orow0 = yw * pitch + xc;
+    const int orow0 = yw * pitch + xc + zero;
     // own rows overlap the tile rows lo .. hi
     auto need = [&](int lo, int hi) { return ry <= hi && ry + R - 1 >= lo; };
-    auto ld = [&](const float *__restrict__ p, int o) {
-        if constexpr (SEAM) return mk(__ldg(p + o), __ldg(p + o + dxc));
-        else return __ldg(reinterpret_cast<const float2 *>(p + o));
+    auto ld = [&](const float *p, int o) {
+        if constexpr (SEAM) return mk(tile2d::ld(p + o), tile2d::ld(p + o + dxc));
+        else return ld2(p + o);
     };
     auto st = [&](float *p, int o, f2 v) {
         if constexpr (SEAM) {
@@ -242,22 +242,19 @@ constexpr int BOTH = 2;
 template <int SET, int M, int P, bool HJ>
 __global__ void __launch_bounds__(32 * NW, 2) k_tile2d(Fused2dArgs<float> a, Geo g, Coef2 c, Tile2dGeo t) {
     extern __shared__ __align__(16) float2 tsm[];
-    // launched while the kernel before it in the stream still runs: nothing is
-    // read or written before that one is done, and the next may come up now
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int zero = dependency_wait();
     const int x0 = (int)(blockIdx.x % t.ntx) * t.tw, y0 = (int)(blockIdx.x / t.ntx) * t.th;
     const int th = min(t.th, g.ny - y0);
     constexpr int HC = TileHalo<M, P, HJ>::HC;
     const bool seam = (g.nx & 1) && (x0 < HC || x0 - HC + 64 > g.nx);
     const bool tm = SET == TM || (SET == BOTH && blockIdx.y == 1);
     if (SET != TM && !tm) {
-        if (!seam) tile_step<TE, M, P, HJ, false>(a, g, c, t.tw, th, x0, y0, tsm);
-        else tile_step<TE, M, P, HJ, true>(a, g, c, t.tw, th, x0, y0, tsm);
+        if (!seam) tile_step<TE, M, P, HJ, false>(a, g, c, t.tw, th, x0, y0, zero, tsm);
+        else tile_step<TE, M, P, HJ, true>(a, g, c, t.tw, th, x0, y0, zero, tsm);
     }
     if (SET != TE && tm) {
-        if (!seam) tile_step<TM, M, P, HJ, false>(a, g, c, t.tw, th, x0, y0, tsm);
-        else tile_step<TM, M, P, HJ, true>(a, g, c, t.tw, th, x0, y0, tsm);
+        if (!seam) tile_step<TM, M, P, HJ, false>(a, g, c, t.tw, th, x0, y0, zero, tsm);
+        else tile_step<TM, M, P, HJ, true>(a, g, c, t.tw, th, x0, y0, zero, tsm);
     }
 }
 

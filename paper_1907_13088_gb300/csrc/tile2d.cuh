@@ -18,6 +18,32 @@ constexpr int R = 8, NW = 8;  // rows per warp, warps per CTA
 __device__ __forceinline__ float up1(float v) { return __shfl_up_sync(FULL, v, 1); }
 __device__ __forceinline__ float dn1(float v) { return __shfl_down_sync(FULL, v, 1); }
 __device__ __forceinline__ f2 sub(f2 a, f2 b) { return fma(b, m1(), a); }
+
+// The kernels are launched while the one before them in the stream still runs
+// (programmatic dependent launch): nothing is read or written before that one is
+// done, and the next may come up from here on.  Returns a zero that the compiler
+// does not know, to go into the load addresses: ld and ld2 may move freely, but
+// not ahead of the wait.  (Not __ldg: the kernel before may write these arrays
+// while this one is already resident, which the read-only path does not allow and
+// the wait does not order.  Plain loads cannot move past the shared-memory stores
+// and spill 12 to 72 bytes.)  What they read must not be written by the kernel.
+__device__ __forceinline__ int dependency_wait() {
+    int zero;
+    asm volatile("griddepcontrol.wait;\n\tmov.s32 %0, 0;" : "=r"(zero)::"memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    return zero;
+}
+__device__ __forceinline__ float ld(const float *p) {
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ f2 ld2(const float *p) {
+    f2 v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 // columns 2t-1 and 2t+2 beside the own pair: f[i-1] + f[i+1]
 __device__ __forceinline__ f2 xsum(f2 v, float l, float r) { return mk(l + v.y, v.x + r); }
 
