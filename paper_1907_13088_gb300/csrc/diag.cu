@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(NT, 2) k_diag3(Geo g, Coef<double> c, double i
     block_partials(v, threadIdx.x, partials + (int64_t)blockIdx.x * NQ);
 }
 
-// 1D
+// One thread per cell: 1D, and 3D grids of one plane that the strips do not fit
 template <typename T, int DIM>
 __global__ void k_diag(Geo g, Coef<double> c, double idx_, double idy_, double idz_, const T *e0, const T *e1,
                        const T *e2, const T *b0, const T *b1, const T *b2, double *partials) {
@@ -369,6 +369,7 @@ int launch_diagnostics(const Geo &g, int dims, const Coef<double> &c, const doub
         double least = 1e300;
         for (int64_t h = 6; h <= 64; ++h) {
             const int64_t nb = (lines * ((len + h - 1) / h) + NT / 32 - 1) / (NT / 32);
+            if (nb * NQ > nparts) continue;
             const double cost = (double)((nb + sms - 1) / sms) * (double)(h + 1);
             if (cost < least) {
                 least = cost;
@@ -376,8 +377,14 @@ int launch_diagnostics(const Geo &g, int dims, const Coef<double> &c, const doub
                 blocks = nb;
             }
         }
-        if (blocks * NQ > nparts || blocks > 2147483647LL) return -1;
-        if (dims == 3)
+        if (blocks > 2147483647LL) return -1;
+        if (blocks == 0) {
+            // no height's partial sums fit the array, which holds one slot per block
+            // of 32 x 8 cells: 3D grids of one plane (one thread per cell there)
+            if (dims != 3) return -1;
+            k_diag<T, 3><<<grid, dim3(BX, BY), 0, s>>>(g, c, ix, iy, iz, E[0], E[1], E[2], B[0], B[1], B[2], partials);
+            blocks = nslots;
+        } else if (dims == 3)
             k_diag3<T><<<(unsigned)blocks, NT, 0, s>>>(g, c, ix, iy, iz, E[0], E[1], E[2], B[0], B[1], B[2], nstrip,
                                                        (int)L, partials);
         else
