@@ -58,13 +58,15 @@ class GaussSourceRun:
 
     # ------------------------------------------------------------------
     def _state(self):
-        """A copy of the grid's state, (E, B) of shape (3, ny, nx) each."""
+        """A copy of the grid's state, (E, B) of shape (3, ny, nx) each.  Two
+        tensors of their own, no views of one: autograd lets a caller edit an
+        output in place only if it is no view of another tensor."""
         g = self.grid
-        out = self.torch.empty((6,) + self.shape[::-1], dtype=g.dtype, device=g.device)
-        csz = g.cells * out.element_size()
-        ptrs = (ctypes.c_void_p * 9)(*[out.data_ptr() + c * csz for c in range(6)], None, None, None)
+        E, B = (self.torch.empty((3,) + self.shape[::-1], dtype=g.dtype, device=g.device) for _ in range(2))
+        csz = g.cells * E.element_size()
+        ptrs = (ctypes.c_void_p * 9)(*[F.data_ptr() + c * csz for F in (E, B) for c in range(3)], None, None, None)
         fmx.check(fmx.fmx_get_fields(g.handle, fmx.FMX_E | fmx.FMX_B, ptrs, fmx.FMX_DEVICE), "fmx_get_fields")
-        return out[:3], out[3:]
+        return E, B
 
     def _setup(self, theta):
         th = np.ascontiguousarray(np.asarray(theta, dtype=np.float64))
