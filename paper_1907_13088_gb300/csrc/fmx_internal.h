@@ -145,12 +145,10 @@ struct ResidentWait {
     long long limit_cycles;
     int lost_arrival;
 };
+// returns the clusters launched, or -1
 template <typename T>
 int launch_resident(const Geo &g, int dims, const Coef<T> &c, const StagedPtrs<T> &P, int nsteps, bool resid, int m,
                     double tol2, int m_max, int jpasses, const ResidentWait &wait, cudaStream_t s);
-// clusters the resident engine launches for a grid of `cells` cells
-template <typename T>
-int resident_clusters(int dims, int64_t cells, bool lost_arrival);
 // CTAs in the cluster the resident kernel launches with (16 where the device
 // runs clusters of 16, else 8)
 template <typename T>

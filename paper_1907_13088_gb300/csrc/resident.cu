@@ -6,9 +6,9 @@
 //
 // The launch is one thread-block cluster (16 CTAs where the device schedules
 // clusters of 16, else 8, one CTA per SM) or, where the arithmetic needs more
-// SMs (FP64 runs at 1/64 of the FP32 rate on this class of part: grids above
-// ~4096 FP64 cells), up to 8 clusters in one cooperative launch (every CTA
-// co-resident).  Each CTA owns a contiguous
+// SMs (FP64 runs at 1/64 of the FP32 rate on this class of part), up to 8 clusters
+// in one cooperative launch (every CTA co-resident; clusters_for has the sizes).
+// Each CTA owns a contiguous
 // range of cells (linear index, x fastest).  Phases are separated by
 //   - one cluster: the cluster's hardware barrier (barrier.cluster
 //     arrive.release / wait.acquire);
@@ -20,11 +20,10 @@
 //     a wait that gives up as soon as another cluster has), then a second
 //     cluster barrier releases the cluster with the leader's verdict.
 // Field data other CTAs wrote is read through L2 (ld.global.cg).  The
-// residual of a sweep is reduced in FP64: warp shuffles, then the warps of a
-// CTA in a fixed order, then every CTA writes its partial into each CTA of
-// its cluster (distributed shared memory) and sums the cluster's partials in
-// rank order; with several clusters each leader publishes its cluster's sum
-// and every thread adds the clusters' sums in cluster order after the grid
+// residual of a sweep is reduced in FP64 by one warp of each CTA in a fixed order
+// (launch_sum): its CTA's values, which it writes into every CTA of the cluster
+// (distributed shared memory), then the cluster's; with several clusters each
+// leader publishes its cluster's sum, and the warp adds those after the grid
 // barrier.  All threads therefore hold bit-identical norms and take the same
 // stop decision: control flow stays uniform and every barrier is reached by
 // every thread (or every wait gives up within its limit).
@@ -427,9 +426,11 @@ __global__ void __launch_bounds__(kNT) k_resident(ResidentArgs<T> a, Geo g) {
 // load and the last store.  (Through L2 a phase took 6.6 us at 64^2, in FP32 as
 // in FP64: about 22 loads of 700 cycles and a barrier that waits for the
 // stores to reach L2.)  Only without a filtered current.
-// us per step (20 steps a call), 64^2: FP64 to 1e-13 (13 sweeps) 119 -> 91.5, FP32 to 1e-5 (5 sweeps)
-// 53 -> 40; 128^2 FP32 (3 sweeps) 59 -> 42.5.  A fixed sweep takes 3.2 us in FP64 (its
-// 26 operations per cell: 2 us) and 0.8 us in FP32.
+// us per step (20 steps a call, either side with the 22 us that a clock query per
+// call then took), 64^2: FP64 to 1e-13 (12 sweeps) 119 -> 91.5, FP32 to 1e-5 (5 sweeps)
+// 53 -> 40; 128^2 FP32 (3 sweeps) 59 -> 42.5; without the query 60.5, 14.4 and 16.1.
+// A fixed sweep takes 3.2 us in FP64 (its 26 operations per cell: 2 us) and 0.8 us in
+// FP32.
 template <typename T>
 __global__ void __launch_bounds__(kNT) k_resident_rows(ResidentArgs<T> a, Geo g, int R) {
     extern __shared__ __align__(16) unsigned char rsm[];
@@ -661,39 +662,66 @@ struct ResidentLauncher {
         static bool r = false;
         return r;
     }
-    // A grid barrier costs ~3 us per phase (an L2 atomic round trip and a
-    // poll); other clusters pay when they take more FP64 work off the cluster's
-    // SMs than that (in FP32 the residual's conversions and squares).  us per
-    // step, Algorithm 1 to 1e-13 in FP64, to 1e-5 in FP32, by clusters: FP64 90^2
-    // 124 (1), 129 (2), 127 (4); 128^2 163 (1), 156 (2), 124 (4), 116 (7); FP32 128^2
-    // 59 (1), 65 (7); 200^2 92 (1), 73 (5); 256^2 112 (2), 88 (4), 82 (7).
-    static int clusters_for(int64_t cells, bool lost) {
+    // Clusters of a launch.  A grid barrier costs ~3 us per phase (an L2 atomic
+    // round trip and a poll) on top of a cluster's; other clusters pay when they
+    // take more work off the cluster's SMs than that.  Where that is depends on
+    // the path: the shared-memory engine (k_resident_rows, one cluster only) is
+    // far ahead of several clusters through L2 until FP64 arithmetic binds it, a
+    // 3D cell has about six times the operations of a 2D one, a 1D cell a few.
+    // us per step by clusters, random fields, 10 steps a call, residual to 1e-13
+    // in FP64 and 1e-5 in FP32 (m = 4 in brackets):
+    //   FP64 3D     16^3 767 (1), 731 (2); 17^3 1084 (1), 798 (2), 751 (3), 687 (4);
+    //               20^3 1438 (1), 1059 (2), 724 (4) [112 (1), 100 (2), 84 (4)];
+    //               22^3 1358 (2), 736 (6)
+    //   FP64 2D     shared memory 80 x 64 318 (1), 480 (2); 90^2 470 (1), 475 (2), 432 (3),
+    //               466 (5); 100^2 513 (1), 523 (3), 473 (5); 128^2 705 (1), 483 (7);
+    //               filtered current 80 x 64 379 (1), 423 (2); 100^2 587 (1), 469 (5)
+    //   FP64 1D     8000 143 (1), 203 (2); 12000 201 (1), 227 (6); 16384 232 (1), 239 (7)
+    //   FP32 2D     shared memory 160^2 54 (1), 94 (7); 200^2 74 (1), 104 (7);
+    //               through L2 256^2 186 (1), 117 (7); filtered 150^2 98 (1), 98 (7)
+    //   FP32 3D     25^3 92 (1), 101 (4); 29^3 124 (1), 103 (7); 32^3 148 (1), 121 (4)
+    //   FP32 1D     20000 66 (1), 74 (5); 40000 111 (1), 85 (5)
+    // FP32 with fixed m stays on one cluster up to 65536 cells whatever the path:
+    // several clusters report a barrier's time-out through a synchronising
+    // read-back, one cluster only enqueues (and can be captured).
+    static int clusters_for(const Geo &g, const ResidentArgs<T> &a) {
         if (coop_refused()) return 1;
-        if (cells <= (sizeof(T) == 8 ? 8192 : 24576)) return 1;
+        const int64_t cells = (int64_t)g.nx * g.ny * g.nz;
+        int64_t one;
+        if (sizeof(T) == 8) one = DIM == 3 ? 4096 : 8192;
+        else one = rows_bytes(g, a) ? cells : (a.resid ? 24576 : 65536);
+        if (cells <= one) return 1;
         const int64_t per_cta = sizeof(T) == 8 ? 128 : 512;
         const int64_t want = (cells + per_cta * cluster() - 1) / (per_cta * cluster());
-        int n = (int)(want < 1 ? 1 : want);
         const int mc = max_clusters();
-        if (n > mc) n = mc;
-        (void)lost;
-        return n;
+        return want < mc ? (int)want : mc;
     }
-    // the shared-memory engine, where the grid takes one cluster and fits it;
-    // false where it does not apply
-    static bool run_rows(const Geo &g, const ResidentArgs<T> &a, int ncl, cudaStream_t s) {
-        if (DIM != 2 || ncl != 1 || a.lost || (a.have_j && a.jpasses > 0)) return false;
-        const int cs = cluster(), R = (g.ny + cs - 1) / cs;
+    static int rows_limit() {  // shared memory of a CTA
         static const int lim = [] {
             int dev = 0, v = 0;
             cudaGetDevice(&dev);
             return cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess ? v : 0;
         }();
+        return lim;
+    }
+    // shared memory per CTA of the shared-memory engine; 0 where it does not apply
+    static size_t rows_bytes(const Geo &g, const ResidentArgs<T> &a) {
+        if (DIM != 2 || a.lost || (a.have_j && a.jpasses > 0)) return 0;
+        const int cs = cluster(), R = (g.ny + cs - 1) / cs;
         const size_t need = (size_t)15 * (R + 2) * g.nx * sizeof(T);
         // half the cluster's CTAs with rows at least; 4 KB for the static part
-        if (2 * ((g.ny + R - 1) / R) < cs || need + 4096 > (size_t)lim) return false;
+        if (2 * ((g.ny + R - 1) / R) < cs || need + 4096 > (size_t)rows_limit()) return 0;
+        return need;
+    }
+    // the shared-memory engine, where the grid takes one cluster and fits it;
+    // false where it does not apply
+    static bool run_rows(const Geo &g, const ResidentArgs<T> &a, int ncl, cudaStream_t s) {
+        const size_t need = ncl == 1 ? rows_bytes(g, a) : 0;
+        if (need == 0) return false;
+        const int cs = cluster(), R = (g.ny + cs - 1) / cs;
         auto k = k_resident_rows<T>;
         static const bool attr =
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim - 4096) == cudaSuccess &&
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_limit() - 4096) == cudaSuccess &&
             (cs <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess);
         if (!attr) {
             cudaGetLastError();
@@ -712,7 +740,9 @@ struct ResidentLauncher {
         cudaGetLastError();
         return false;
     }
+    // ncl receives the launch's clusters
     static cudaError_t run(const Geo &g, const ResidentArgs<T> &a, int &ncl, cudaStream_t s) {
+        ncl = clusters_for(g, a);
         if (run_rows(g, a, ncl, s)) return cudaSuccess;
         const int cs = cluster();
         cudaLaunchConfig_t cfg = {};
@@ -749,13 +779,6 @@ int resident_cluster_size(int dims) {
 }
 
 template <typename T>
-int resident_clusters(int dims, int64_t cells, bool lost_arrival) {
-    return dims == 3 ? ResidentLauncher<T, 3>::clusters_for(cells, lost_arrival)
-                     : (dims == 2 ? ResidentLauncher<T, 2>::clusters_for(cells, lost_arrival)
-                                  : ResidentLauncher<T, 1>::clusters_for(cells, lost_arrival));
-}
-
-template <typename T>
 int launch_resident(const Geo &g, int dims, const Coef<T> &c, const StagedPtrs<T> &P, int nsteps, bool resid, int m,
                     double tol2, int m_max, int jpasses, const ResidentWait &wait, cudaStream_t s) {
     ResidentArgs<T> a;
@@ -770,8 +793,7 @@ int launch_resident(const Geo &g, int dims, const Coef<T> &c, const StagedPtrs<T
     a.have_j = P.J[0] != nullptr;
     a.limit = wait.limit_cycles;
     a.lost = wait.lost_arrival ? 1 : 0;
-    const int64_t cells = (int64_t)g.nx * g.ny * g.nz;
-    int ncl = resident_clusters<T>(dims, cells, a.lost != 0);
+    int ncl = 1;
     cudaError_t e = dims == 3 ? ResidentLauncher<T, 3>::run(g, a, ncl, s)
                               : (dims == 2 ? ResidentLauncher<T, 2>::run(g, a, ncl, s)
                                            : ResidentLauncher<T, 1>::run(g, a, ncl, s));
@@ -780,8 +802,6 @@ int launch_resident(const Geo &g, int dims, const Coef<T> &c, const StagedPtrs<T
 
 template int resident_cluster_size<float>(int);
 template int resident_cluster_size<double>(int);
-template int resident_clusters<float>(int, int64_t, bool);
-template int resident_clusters<double>(int, int64_t, bool);
 template int launch_resident<float>(const Geo &, int, const Coef<float> &, const StagedPtrs<float> &, int, bool, int,
                                     double, int, int, const ResidentWait &, cudaStream_t);
 template int launch_resident<double>(const Geo &, int, const Coef<double> &, const StagedPtrs<double> &, int, bool,
