@@ -409,17 +409,14 @@ fmx_status filter_in_place(fmx_grid *g, T *f, int passes) {
     return check_launch(g, "filter kernel launch");
 }
 
-// The same on several components (at most 6) at once.  The scratch is what no
-// state lives in between steps: the fused engine's other state set, the staged
-// layout's dEa and dEb elsewhere.
+// The same on several components (at most 6) at once, through workspace only: the
+// spare array tmp in 2D, dEa and dEb (which hold nothing between steps) elsewhere.
 template <typename T>
 fmx_status filter_fields(fmx_grid *g, T *const f[], int n, int passes) {
     T *scratch[6];
-    for (int q = 0; q < 6; ++q) {
-        if (g->engine == FMX_ENGINE_FUSED) scratch[q] = (T *)(q < 3 ? g->buf.E[1 - g->cur][q] : g->buf.B[1 - g->cur][q - 3]);
-        else scratch[q] = (T *)(q < 3 ? g->dEa[q] : g->dEb[q - 3]);
-    }
-    const int nl = passes > 0 ? fmx::launch_filter_fields<T>(g->geo, g->p.dims, passes, n, f, scratch, g->stream) : 0;
+    for (int q = 0; q < 6; ++q) scratch[q] = (T *)(q < 3 ? g->dEa[q] : g->dEb[q - 3]);
+    const int nl =
+        passes > 0 ? fmx::launch_filter_fields<T>(g->geo, g->p.dims, passes, n, f, scratch, (T *)g->tmp, g->stream) : 0;
     if (nl) {
         g->launches += nl;
         return check_launch(g, "filter kernel launch");

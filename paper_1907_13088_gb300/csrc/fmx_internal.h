@@ -73,12 +73,14 @@ int64_t staged_partial_slots(const Geo &g);
 template <typename T>
 int launch_filter_pass(const Geo &g, int dims, const T *in, T *out, int axis, cudaStream_t s);
 
-// `passes` binomial passes along every active axis of n (at most 6) components,
-// in place through as many scratch arrays, in two launches.  Returns 0 (nothing
-// launched) where the kernels are not instantiated (passes above 3, or a grid
-// beyond the flattened launch limits).
+// `passes` binomial passes along every active axis of n (at most 6) components, in
+// place, in two launches: through as many scratch arrays (1D, 3D), or through the
+// one array `spare` (2D; in parts where it has not room for all).  Returns the
+// launches, 0 (nothing launched) where the kernels are not instantiated (passes
+// above 3, a grid beyond the flattened launch limits, or too small for spare).
 template <typename T>
-int launch_filter_fields(const Geo &g, int dims, int passes, int n, T *const f[], T *const scratch[], cudaStream_t s);
+int launch_filter_fields(const Geo &g, int dims, int passes, int n, T *const f[], T *const scratch[], T *spare,
+                         cudaStream_t s);
 
 template <typename T>
 int launch_staged_source(const Geo &g, int dims, const Coef<T> &c, const StagedPtrs<T> &p,

@@ -13,6 +13,8 @@
 //   that differentiates along them and alpha becomes 1 (Secs. 2.2.2-2.2.3).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "fmx_internal.h"
 #include "stencil.cuh"
 
@@ -58,13 +60,11 @@ __global__ void k_filter_pass(Geo g, const T *__restrict__ in, T *__restrict__ o
     out[idx] = T(0.25) * f(p, -dx, -dy, -dz) + T(0.5) * f(p, 0, 0, 0) + T(0.25) * f(p, dx, dy, dz);
 }
 
-// Binomial filter of several components at once, P passes along every axis
-// in two launches: the x (3D: x and y) taps from the fields into scratch, the
-// last axis' taps back (1D: copied back).  The P passes of one axis are its
-// (2P+1)-tap binomial, and P = 1 rounds as the single passes do.  Bound by the
-// launches and index arithmetic of a pass over one component at a time before
-// (12 launches for E and B in 2D; 1536 x 1200 FP32, P = 1: 12 x 10 us, now
-// 35 + 33 us, launched cold).
+// Binomial filter of several components at once, P passes along every axis in
+// two launches.  The P passes of one axis are its (2P+1)-tap binomial, and P = 1
+// rounds as the single passes do.  2D: in place, tile by tile (below).  1D and 3D:
+// the x (3D: x and y) taps from the fields into scratch, the last axis' taps back
+// (1D: copied back).
 struct FilterSet {
     const void *in[6];
     void *out[6];
@@ -84,13 +84,161 @@ __device__ __forceinline__ T filter_taps(const T *v) {
     return s;
 }
 
+// 2D, in place: a CTA holds a tile of at most 64 x 64 cells in shared memory, with
+// a halo of P cells that the launch before it saved in ring (a tile's cells are
+// written by its own CTA only, once all of them are loaded).  So the filter takes
+// the workspace's one spare component array and none of the caller's others.  A
+// grid of one tile is its own halo: one launch, ring = nullptr.
+// FP32 is bound by memory: each cell is read and written once, and the halos (P =
+// 1: 6%).  FP64 is bound by its 2 (2P + 1) operations per cell, which is why the x
+// taps are evaluated once per row of the tile (9% more rows than cells at P = 3)
+// and small grids are cut into smaller tiles, over more SMs.
+// ring_size is how much of it a tile of a component takes, ring_cell the cell of
+// its element e: P rows below and above with their corners, then P columns left
+// and right.
+constexpr int FT = 64, FNT = 256;  // tile, threads
+__host__ __device__ constexpr int ring_size(int P, int tw, int th) { return 2 * P * (tw + 2 * P) + 2 * P * th; }
+template <int P>
+__device__ __forceinline__ void ring_cell(int e, int tw, int th, int &col, int &row) {
+    const int w = tw + 2 * P;
+    if (e < 2 * P * w) {
+        const int r = e / w;
+        col = e % w - P;
+        row = r < P ? r - P : th + r - P;
+    } else {
+        e -= 2 * P * w;
+        const int k = e % (2 * P);
+        col = k < P ? k - P : tw + k - P;
+        row = e / (2 * P);
+    }
+}
+struct FilterTiles {
+    int tw, th, ntx, h;  // tile, tiles along x, ring elements per tile
+};
+template <typename T>
+__device__ __forceinline__ T wrapped(const Geo &g, const T *in, int x, int y) {
+    while (x < 0) x += g.nx;
+    while (x >= g.nx) x -= g.nx;
+    while (y < 0) y += g.ny;
+    while (y >= g.ny) y -= g.ny;
+    return in[(int64_t)y * g.pitch + x];
+}
+template <typename T, int P>
+__global__ void __launch_bounds__(FNT) k_filter_halo(Geo g, const __grid_constant__ FilterSet f, FilterTiles t, T *ring) {
+    const T *in = (const T *)f.in[blockIdx.y];
+    const int x0 = (int)(blockIdx.x % t.ntx) * t.tw, y0 = (int)(blockIdx.x / t.ntx) * t.th;
+    const int tw = min(t.tw, g.nx - x0), th = min(t.th, g.ny - y0);
+    T *out = ring + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * t.h;
+    for (int e = threadIdx.x; e < ring_size(P, tw, th); e += blockDim.x) {
+        int col, row;
+        ring_cell<P>(e, tw, th, col, row);
+        out[e] = wrapped(g, in, x0 + col, y0 + row);
+    }
+}
+template <typename T, int P>
+__global__ void __launch_bounds__(FNT) k_filter_tile(Geo g, const __grid_constant__ FilterSet f, FilterTiles t, const T *ring) {
+    constexpr int W = FT + 2 * P;  // shared row
+    __shared__ T sm[W * W];
+    const int x0 = (int)(blockIdx.x % t.ntx) * t.tw, y0 = (int)(blockIdx.x / t.ntx) * t.th;
+    const int tw = min(t.tw, g.nx - x0), th = min(t.th, g.ny - y0);
+    // columns of the tile over 32 or 64 threads, its rows over groups of them
+    const int cols = t.tw <= 32 ? 32 : 64, groups = FNT / cols, col = threadIdx.x % cols, grp = threadIdx.x / cols;
+    T *own = (T *)f.out[blockIdx.y] + (int64_t)y0 * g.pitch + x0 + col;
+    const T *halo = ring + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * t.h;
+#pragma unroll
+    for (int i = 0; i < FT / 4; ++i) {
+        const int r = i * groups + grp;
+        if (r < th && col < tw) sm[(r + P) * W + col + P] = own[r * g.pitch];
+    }
+    for (int e = threadIdx.x; e < ring_size(P, tw, th); e += FNT) {
+        int c, r;
+        ring_cell<P>(e, tw, th, c, r);
+        sm[(r + P) * W + c + P] = ring ? halo[e] : wrapped(g, (const T *)f.in[blockIdx.y], c, r);
+    }
+    __syncthreads();
+    // x taps, a row per warp, in place
+    const int lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < th + 2 * P; r += FNT / 32) {
+        T *row = sm + r * W + lane;
+        const T a = lane < tw ? filter_taps<T, P>(row) : T(0), b = lane + 32 < tw ? filter_taps<T, P>(row + 32) : T(0);
+        __syncwarp();
+        if (lane < tw) row[P] = a;
+        if (lane + 32 < tw) row[32 + P] = b;
+    }
+    __syncthreads();
+    // y taps, up to 16 rows of a column per thread
+    const int run = (th + groups - 1) / groups, r0 = grp * run, n = min(run, th - r0) + 2 * P;
+    if (col >= tw || r0 >= th) return;
+    const T *in = sm + r0 * W + col + P;
+    T *o = own + r0 * g.pitch;
+    T w[2 * P + 1];
+#pragma unroll
+    for (int r = 0; r < FT / 4 + 2 * P; ++r) {
+        if (r >= n) break;
+#pragma unroll
+        for (int k = 0; k < 2 * P; ++k) w[k] = w[k + 1];
+        w[2 * P] = in[r * W];
+        if (r >= 2 * P) o[(r - 2 * P) * g.pitch] = filter_taps<T, P>(w);
+    }
+}
+
+// As many of the n components at a time as the spare array (g.plane elements) has
+// room for; 0 where it has room for none.  Tiles shrink from 64 x 64 to 16 x 16 while
+// there are fewer than two per SM and the halos of all n components still fit.
+template <typename T, int P>
+int filter_tiles(const Geo &g, int n, T *const f[], T *spare, cudaStream_t s) {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
+    }();
+    FilterTiles t{};
+    int64_t tiles = 0, fit = 0;
+    FilterSet a{};
+    if (g.nx <= FT && g.ny <= FT) {
+        for (int q = 0; q < n; ++q) a.in[q] = a.out[q] = f[q];
+        t = FilterTiles{g.nx, g.ny, 1, 0};
+        k_filter_tile<T, P><<<dim3(1, n), FNT, 0, s>>>(g, a, t, nullptr);
+        return 1;
+    }
+    for (int lx = FT, ly = FT; lx >= 16 && ly >= 16;) {
+        const auto even = [](int len, int lim) { return (len + (len + lim - 1) / lim - 1) / ((len + lim - 1) / lim); };
+        FilterTiles c;
+        c.tw = even(g.nx, lx);
+        c.th = even(g.ny, ly);
+        c.ntx = (g.nx + c.tw - 1) / c.tw;
+        c.h = ring_size(P, c.tw, c.th);
+        const int64_t ct = (int64_t)c.ntx * ((g.ny + c.th - 1) / c.th), cf = g.plane / (ct * c.h);
+        if (tiles > 0 && cf < n) break;
+        t = c;
+        tiles = ct;
+        fit = cf;
+        if (tiles * n >= 2 * sms || fit < n) break;
+        if (c.th >= c.tw) ly = (c.th + 1) / 2;
+        else lx = (c.tw + 1) / 2;
+    }
+    if (fit < 1) return 0;
+    const int parts = (int)((n + fit - 1) / fit), per = (n + parts - 1) / parts;
+    int launches = 0;
+    for (int q0 = 0; q0 < n; q0 += per) {
+        const int m = n - q0 < per ? n - q0 : per;
+        for (int q = 0; q < m; ++q) a.in[q] = a.out[q] = f[q0 + q];
+        const dim3 grid((unsigned)tiles, m);
+        k_filter_halo<T, P><<<grid, FNT, 0, s>>>(g, a, t, spare);
+        k_filter_tile<T, P><<<grid, FNT, 0, s>>>(g, a, t, spare);
+        launches += 2;
+    }
+    return launches;
+}
+
 constexpr int FR = 16;  // rows per thread
 template <typename T, int P, bool XY>
-__global__ void __launch_bounds__(BX *BY) k_filter_in_plane(Geo g, FilterSet f, int nbx, int nby) {
+__global__ void __launch_bounds__(BX *BY) k_filter_in_plane(Geo g, const __grid_constant__ FilterSet f, int nbx, int nby) {
     const T *__restrict__ in = (const T *)f.in[blockIdx.y];
     T *__restrict__ out = (T *)f.out[blockIdx.y];
     const unsigned bxy = blockIdx.x / nbx;
-    const int x = (int)(blockIdx.x % nbx) * BX + threadIdx.x, y0 = (int)(bxy % nby) * (BY * FR) + threadIdx.y * FR;
+    const int x = (int)(blockIdx.x % nbx) * BX + threadIdx.x;
+    const int y0 = ((int)(bxy % nby) * blockDim.y + threadIdx.y) * FR;
     const int64_t z = (int64_t)(bxy / nby) * g.plane;
     if (x >= g.nx || y0 >= g.ny) return;
     constexpr int H = XY ? P : 0;
@@ -135,12 +283,13 @@ __global__ void __launch_bounds__(BX *BY) k_filter_in_plane(Geo g, FilterSet f, 
 // `ostride` apart.  P = 0 copies.
 constexpr int FS = 16;  // elements per thread
 template <typename T, int P>
-__global__ void __launch_bounds__(BX *BY) k_filter_last(Geo g, FilterSet f, int n, int64_t stride, int64_t ostride,
-                                                        int nbx, int nseg) {
+__global__ void __launch_bounds__(BX *BY) k_filter_last(Geo g, const __grid_constant__ FilterSet f, int n, int64_t stride,
+                                                        int64_t ostride, int nbx, int nseg) {
     const T *__restrict__ in = (const T *)f.in[blockIdx.y];
     T *__restrict__ out = (T *)f.out[blockIdx.y];
     const unsigned rest = blockIdx.x / nbx;
-    const int x = (int)(blockIdx.x % nbx) * BX + threadIdx.x, j0 = ((int)(rest % nseg) * BY + threadIdx.y) * FS;
+    const int x = (int)(blockIdx.x % nbx) * BX + threadIdx.x;
+    const int j0 = ((int)(rest % nseg) * blockDim.y + threadIdx.y) * FS;
     if (x >= g.nx || j0 >= n) return;
     const int64_t o = (int64_t)(rest / nseg) * ostride + x;
     int j = j0 - P;
@@ -175,16 +324,17 @@ void filter_two(const Geo &g, int dims, int n, T *const f[], T *const scratch[],
         a.out[q] = scratch[q];
         b.in[q] = scratch[q];
     }
-    const int nbx = (g.nx + BX - 1) / BX, nby = (g.ny + BY * FR - 1) / (BY * FR);
-    const dim3 ga((unsigned)((int64_t)nbx * nby * g.nz), n), blk(BX, BY);
-    if (dims == 3) k_filter_in_plane<T, P, true><<<ga, blk, 0, s>>>(g, a, nbx, nby);
-    else k_filter_in_plane<T, P, false><<<ga, blk, 0, s>>>(g, a, nbx, nby);
+    const dim3 ka(BX, BY);
+    const int nbx = (g.nx + BX - 1) / BX, nby = (g.ny + ka.y * FR - 1) / (ka.y * FR);
+    const dim3 ga((unsigned)((int64_t)nbx * nby * g.nz), n);
+    if (dims == 3) k_filter_in_plane<T, P, true><<<ga, ka, 0, s>>>(g, a, nbx, nby);
+    else k_filter_in_plane<T, P, false><<<ga, ka, 0, s>>>(g, a, nbx, nby);
     const int len = dims == 3 ? g.nz : g.ny, others = dims == 3 ? g.ny : 1;
-    const int nseg = (len + BY * FS - 1) / (BY * FS);
+    const dim3 kb(BX, BY);
+    const int nseg = (len + kb.y * FS - 1) / (kb.y * FS);
     const dim3 gb((unsigned)((int64_t)nbx * nseg * others), n);
-    const int64_t st = dims == 3 ? g.plane : g.pitch;
-    if (dims == 1) k_filter_last<T, 0><<<gb, blk, 0, s>>>(g, b, len, st, g.pitch, nbx, nseg);
-    else k_filter_last<T, P><<<gb, blk, 0, s>>>(g, b, len, st, g.pitch, nbx, nseg);
+    if (dims == 3) k_filter_last<T, P><<<gb, kb, 0, s>>>(g, b, len, g.plane, g.pitch, nbx, nseg);
+    else k_filter_last<T, 0><<<gb, kb, 0, s>>>(g, b, len, g.pitch, g.pitch, nbx, nseg);
 }
 
 template <typename T, int DIM>
@@ -409,14 +559,21 @@ int launch_filter_pass(const Geo &g, int dims, const T *in, T *out, int axis, cu
 }
 
 template <typename T>
-int launch_filter_fields(const Geo &g, int dims, int passes, int n, T *const f[], T *const scratch[], cudaStream_t s) {
+int launch_filter_fields(const Geo &g, int dims, int passes, int n, T *const f[], T *const scratch[], T *spare,
+                         cudaStream_t s) {
     // flattened launch grids of at most 2^31 - 1 blocks
     const double blocks = (double)((g.nx + BX - 1) / BX) * (double)g.ny * (double)g.nz;
     if (n < 1 || n > 6 || blocks > 2147483647.0) return 0;
+    auto run = [&](auto p) {
+        constexpr int P = decltype(p)::value;
+        if (dims == 2) return filter_tiles<T, P>(g, n, f, spare, s);
+        filter_two<T, P>(g, dims, n, f, scratch, s);
+        return 2;
+    };
     switch (passes) {
-        case 1: filter_two<T, 1>(g, dims, n, f, scratch, s); return 2;
-        case 2: filter_two<T, 2>(g, dims, n, f, scratch, s); return 2;
-        case 3: filter_two<T, 3>(g, dims, n, f, scratch, s); return 2;
+        case 1: return run(std::integral_constant<int, 1>());
+        case 2: return run(std::integral_constant<int, 2>());
+        case 3: return run(std::integral_constant<int, 3>());
     }
     return 0;
 }
@@ -514,7 +671,7 @@ int launch_faraday(const Geo &g, int dims, const Coef<T> &c, T *const E[3], T *c
 
 #define FMX_INST(T)                                                                                           \
     template int launch_filter_pass<T>(const Geo &, int, const T *, T *, int, cudaStream_t);                  \
-    template int launch_filter_fields<T>(const Geo &, int, int, int, T *const[], T *const[], cudaStream_t);    \
+    template int launch_filter_fields<T>(const Geo &, int, int, int, T *const[], T *const[], T *, cudaStream_t); \
     template int launch_staged_source<T>(const Geo &, int, const Coef<T> &, const StagedPtrs<T> &,            \
                                          const T *const[3], cudaStream_t, bool);                              \
     template int launch_staged_sweep<T>(const Geo &, int, const Coef<T> &, const StagedPtrs<T> &,             \
