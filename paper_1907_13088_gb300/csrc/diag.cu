@@ -355,9 +355,10 @@ int launch_diagnostics(const Geo &g, int dims, const Coef<double> &c, const doub
     if (nslots * NQ > nparts) return -1;
     const double ix = 1.0 / d[0], iy = 1.0 / d[1], iz = 1.0 / d[2];
     if (dims > 1) {
-        // strips of 30 columns, segments of 6 to 64 rows (2D) or planes (3D), the
+        // strips of 30 columns, segments of 1 to 64 rows (2D) or planes (3D), the
         // height at which the fullest SM has the least to do (the first row of a
-        // segment costs about one row more)
+        // segment costs about one row more).  On grids that leave SMs free the lowest
+        // that the partial sums' array holds: a warp's rows follow one another
         const int nstrip = (g.nx + DW - 1) / DW, len = dims == 3 ? g.nz : g.ny;
         const int64_t lines = (int64_t)nstrip * (dims == 3 ? g.ny : 1);
         static const int sms = [] {
@@ -367,7 +368,7 @@ int launch_diagnostics(const Geo &g, int dims, const Coef<double> &c, const doub
         }();
         int64_t L = 6, blocks = 0;
         double least = 1e300;
-        for (int64_t h = 6; h <= 64; ++h) {
+        for (int64_t h = 1; h <= 64; ++h) {
             const int64_t nb = (lines * ((len + h - 1) / h) + NT / 32 - 1) / (NT / 32);
             if (nb * NQ > nparts) continue;
             const double cost = (double)((nb + sms - 1) / sms) * (double)(h + 1);

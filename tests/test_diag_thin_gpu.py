@@ -1,6 +1,6 @@
 """Diagnostics of 3D grids of one plane, whose strips of 30 columns are more than
-the 32-column blocks that the partial sums' buffer is sized by, against the FP64
-oracle."""
+the 32-column blocks that the partial sums' buffer is sized by, and of grids whose
+segments go down to one row or plane, against the FP64 oracle."""
 import numpy as np
 import pytest
 
@@ -31,7 +31,7 @@ def _close(a, b):
 def test_diagnostics_of_one_plane(fmx, shape, f64):
     dt = np.float64 if f64 else np.float32
     E, B, _ = (a.astype(dt) for a in synth.random_fields(shape, 461))
-    kw = dict(courant=0.7, m=3, d=(1.0, 0.8, 1.2))
+    kw = dict(courant=0.7, m=3, d=(1.0, 0.8, 1.2)[:len(shape)])
     g = fmx.Grid(shape, precision=1 if f64 else 0, with_current=False, **kw)
     g.set_fields(E, B)
     d = g.diagnostics()
@@ -42,3 +42,9 @@ def test_diagnostics_of_one_plane(fmx, shape, f64):
     assert _close(d["w_scheme"], ws) and _close(d["w_plain"], wp)
     assert _close(d["divb_max"], np.max(np.abs(db))) and _close(d["divb_l2"], np.linalg.norm(db))
     assert _close(d["gauss_max"], np.max(np.abs(ge))) and _close(d["gauss_l2"], np.linalg.norm(ge))
+
+
+@pytest.mark.parametrize("f64", [True, False])
+@pytest.mark.parametrize("shape", [(64, 64), (3000, 5), (33, 2), (29, 1), (1, 1), (100, 3, 2), (20, 30, 7)])
+def test_diagnostics_of_few_rows(fmx, shape, f64):
+    test_diagnostics_of_one_plane(fmx, shape, f64)
