@@ -461,10 +461,11 @@ struct Launcher {
             // the CTAs of one SM share its FP64 arithmetic: the segment count with
             // the least (CTAs of the fullest SM) x (rows each computes, about 6
             // beyond its own), c resident CTAs leaving 1/(2c) of their latencies open
+            // (each height once: n segments, then the fewest whose rows are fewer)
             double least = 1e300;
-            for (int n = 1; n <= g.ny; ++n) {
-                const int rows = (g.ny + n - 1) / n;
-                if (n > 1 && (rows < 8 || (long long)sh.strips * n > 64LL * sms)) break;  // finer only adds rows
+            for (int n = 1, rows; n <= g.ny; n = rows > 1 ? (g.ny - 1) / (rows - 1) + 1 : g.ny + 1) {
+                rows = (g.ny + n - 1) / n;
+                if (n > 1 && (long long)sh.strips * n > 64LL * sms) break;  // finer only adds rows
                 const long long k = ((long long)sh.strips * ((g.ny + rows - 1) / rows) + sms - 1) / sms;
                 const double load = (double)(k / bps) * (bps + 0.5) + (k % bps ? (double)(k % bps) + 0.5 : 0.0);
                 if (load * (rows + 6) < least) {
