@@ -21,25 +21,28 @@ namespace {
 
 constexpr int TY = 8, NTH = 32 * TY, RH = TY + 2;  // pair kernels: rows of the tile, threads, rows with halo
 
-// planes a segment marches over.  The CTAs on one SM share its arithmetic, so a
-// launch takes about the CTAs of the fullest SM times the planes each marches
-// (two more than it writes), and c of them resident at a time leave their
-// latencies open, which a factor 1 + lat/c stands for (0.5; 0.6 for the CTAs of
-// two warps, or 64^3 FP64 would leave one of them on an SM: 450 us a step, 300 so); the segment height
-// with the least product, 4 to 64 planes, is taken (128 x 128 x 96 FP64 sweep, CTAs
-// of four warps: 24 planes, one CTA on each of 128 SMs, 270 us; 7 planes, 448
-// CTAs, 250 us).  tiles: CTAs per segment; res: CTAs an SM holds.
-int zseg_for(int nz, long long tiles, int res, double lat) {
+int sm_count() {
     static const int sms = [] {
         int dev = 0, v = 0;
         cudaGetDevice(&dev);
         return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
     }();
+    return sms;
+}
+
+// planes a segment marches over.  The CTAs on one SM share its arithmetic, so a
+// launch takes about the CTAs of the fullest SM times the planes each marches
+// (two more than it writes), and c of them resident at a time leave their
+// latencies open, which a factor 1 + lat/c stands for (0.5; 0.6 for the CTAs of
+// two warps, or 64^3 FP64 would leave one of them on an SM: 450 us a step, 300 so); the segment height
+// with the least product, 1 to 64 planes, is taken (128 x 128 x 96 FP64 sweep, CTAs
+// of four warps: 24 planes, one CTA on each of 128 SMs, 270 us; 7 planes, 448
+// CTAs, 250 us).  tiles: CTAs per segment; res: CTAs an SM holds.
+int zseg_for(int nz, long long tiles, int res, double lat) {
+    const int sms = sm_count();
     int best = 1;
     double least = 1e300;
-    for (int nseg = (nz + 63) / 64; nseg <= nz; ++nseg) {
-        const int z = (nz + nseg - 1) / nseg;
-        if (z < 4 && nseg > 1) break;
+    for (int z = nz < 64 ? nz : 64; z >= 1; --z) {
         const long long n = (tiles * ((nz + z - 1) / z) + sms - 1) / sms;  // CTAs of the fullest SM
         // rounds of res resident CTAs, then the rest
         const double load = (double)(n / res) * (res + lat) + (n % res ? (double)(n % res) + lat : 0.0);
@@ -85,13 +88,18 @@ __device__ __forceinline__ void cp_async_wait() {
 // source 52 against about 150.  128 x 128 x 96 FP64, 16 rows: sweep 685 -> 242 us,
 // source 627 -> 231 us (their operations take 213 and 189 us at the FMA rate that
 // fmx_fma_peak measures); 201 x 150 x 99 FP32: sweep 53 -> 33 us, source 68 -> 38 us.
-constexpr int CX = 32, CR = 4, CW = 2, CROWS = CR * CW, CNT = 32 * CW;
-constexpr int CPW = CX + 2, CPL = CPW * (CROWS + 2);  // row and plane of the tile with its halo
-constexpr int CCP = (CPL + CNT - 1) / CNT;             // copies of a component plane per thread
+//
+// The FP64 units sit one to a quarter of an SM, and a warp's rows follow one another
+// on its own: with fewer warps than a quarter of them (grids of few cells, or of one
+// or two planes) the rows are given to more warps, CR = 1 row per thread (one_row).
+constexpr int CX = 32, CW = 2, CNT = 32 * CW;
+constexpr int CPW = CX + 2;                                               // row of the tile with its halo
+__host__ __device__ constexpr int cpl(int CR) { return CPW * (CR * CW + 2); }  // plane with its halo
 
 // the copies of the tile's planes: plane z0 - 1 + i into ring slot i mod RS
-template <typename T, int N, int RS>
+template <typename T, int N, int RS, int CR>
 struct ColPlanes {
+    static constexpr int CPL = cpl(CR), CCP = (CPL + CNT - 1) / CNT;  // copies of a component plane per thread
     int off[CCP];  // in-plane offsets of the thread's elements
     int64_t base;  // element offset of the plane copied next, wrapped into [0, n_z)
     int slot;
@@ -118,15 +126,31 @@ struct ColPlanes {
     }
 };
 
+// the rows of a thread in turn; left: rows of the grid from its first on (the
+// warp's, so the branch is uniform).  Rows past the grid are skipped, but not with
+// a test per row where there are none: the rows' operations interleave.  FP64 only:
+// FP32 arithmetic does not bind, and the second body costs 1% (201 x 150 x 99).
+template <int CR, typename F>
+__device__ __forceinline__ void each_row(int left, const F &row) {
+    if (left >= CR) {
+#pragma unroll
+        for (int r = 0; r < CR; ++r) row(r);
+    } else {
+#pragma unroll
+        for (int r = 0; r < CR - 1; ++r)
+            if (r < left) row(r);
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ T d2s(T a, T v, T b) { return (a + b) - T(2) * v; }  // a - 2 v + b
 
 // out = dEp + A in, or with UPD E = E + dEp + A in (E in place)
 constexpr int SWEEP1_RS = 4;
-template <typename T, bool UPD>
+template <typename T, bool UPD, int CR>
 __global__ void __launch_bounds__(CNT, 6) k3_sweep1(Geo g, Coef<T> c, const T *p0, const T *p1, const T *p2, const T *i0,
                                                  const T *i1, const T *i2, T *o0, T *o1, T *o2, int zseg) {
-    constexpr int RS = SWEEP1_RS;
+    constexpr int RS = SWEEP1_RS, CROWS = CR * CW, CPL = cpl(CR);
     extern __shared__ __align__(16) unsigned char m3raw[];
     T *ring = reinterpret_cast<T *>(m3raw);  // [RS][3][CPL]
     const T *in[3] = {i0, i1, i2};
@@ -136,7 +160,7 @@ __global__ void __launch_bounds__(CNT, 6) k3_sweep1(Geo g, Coef<T> c, const T *p
     const int x0 = blockIdx.x * CX, y0 = blockIdx.y * CROWS;
     const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
     const int np = z1 - z0 + 2;  // input planes z0-1 .. z1
-    ColPlanes<T, 3, RS> cp;
+    ColPlanes<T, 3, RS, CR> cp;
     cp.init(g, x0, y0, z0 - 1);
     auto issue = [&](int i) {
         if (i < np) cp.issue_next(ring, in, g);
@@ -187,8 +211,7 @@ __global__ void __launch_bounds__(CNT, 6) k3_sweep1(Geo g, Coef<T> c, const T *p
             d_0 = d2s(V(2, -1, 0), ez_0, er0);
             zx_0 = ez_0 + c.c6 * d_0;
         }
-#pragma unroll
-        for (int r = 0; r < CR; ++r) {
+        auto row = [&](int r) {
             // Ex: P = Dbar_yy Ex, X = Dbar_x (Ex + P/6), Gp = Dbar_x Dbar_y Ex
             const T ex_p = V(0, 0, r + 1), b_p = ex_p - V(0, -1, r + 1);
             const T P = d2s(ex_p, ex_0, ex_m), X = b_0 + c.c6 * d2s(b_p, b_0, b_m), Gp = b_p - b_0;
@@ -222,7 +245,8 @@ __global__ void __launch_bounds__(CNT, 6) k3_sweep1(Geo g, Coef<T> c, const T *p
             ex_m = ex_0, ex_0 = ex_p, b_m = b_0, b_0 = b_p;
             a_m = a_0, yp_m = yp_0;
             ez_m = ez_0, ez_0 = ez_p, c_m = c_0, c_0 = c_p, d_m = d_0, d_0 = d_p, zx_0 = zx_p;
-        }
+        };
+        each_row<CR>(sizeof(T) == 8 ? g.ny - y : CR, row);
         if (i >= 2) cell += g.plane;
     }
     cp_async_wait<0>();
@@ -232,10 +256,10 @@ __global__ void __launch_bounds__(CNT, 6) k3_sweep1(Geo g, Coef<T> c, const T *p
 // (PASSES = 1) or none (PASSES = 0); HJ: a current is bound.  The terms of
 // curl_plane_terms below, per row.
 constexpr int SOURCE1_RS = 3;
-template <typename T, int PASSES, bool HJ>
+template <typename T, int PASSES, bool HJ, int CR>
 __global__ void __launch_bounds__(CNT) k3_source1(Geo g, Coef<T> c, const T *b0, const T *b1, const T *b2, const T *j0,
                                                   const T *j1, const T *j2, T *o0, T *o1, T *o2, int zseg) {
-    constexpr int RS = SOURCE1_RS, N = HJ ? 6 : 3;
+    constexpr int RS = SOURCE1_RS, N = HJ ? 6 : 3, CROWS = CR * CW, CPL = cpl(CR);
     extern __shared__ __align__(16) unsigned char m3raw[];
     T *ring = reinterpret_cast<T *>(m3raw);  // [RS][N][CPL]
     const T *src[6] = {b0, b1, b2, j0, j1, j2};
@@ -244,7 +268,7 @@ __global__ void __launch_bounds__(CNT) k3_source1(Geo g, Coef<T> c, const T *b0,
     const int x0 = blockIdx.x * CX, y0 = blockIdx.y * CROWS;
     const int z0 = blockIdx.z * zseg, z1 = min(z0 + zseg, g.nz);
     const int np = z1 - z0 + 2;  // input planes z0-1 .. z1
-    ColPlanes<T, N, RS> cp;
+    ColPlanes<T, N, RS, CR> cp;
     cp.init(g, x0, y0, z0 - 1);
     auto issue = [&](int i) {
         if (i < np) cp.issue_next(ring, src, g);
@@ -289,8 +313,7 @@ __global__ void __launch_bounds__(CNT) k3_source1(Geo g, Coef<T> c, const T *b0,
                 s_0[q] = jr(q, 0);
             }
         }
-#pragma unroll
-        for (int r = 0; r < CR; ++r) {
+        auto row = [&](int r) {
             const T by_p = V(1, 0, r + 1), u_p = by_p - V(1, -1, r + 1);
             const T U = by_0 + c.c6 * d2s(by_p, by_0, by_m), Ux = u_0 + c.c6 * d2s(u_p, u_0, u_m);
             const T W = wx(r), Wy = W - w_m;
@@ -341,7 +364,8 @@ __global__ void __launch_bounds__(CNT) k3_source1(Geo g, Coef<T> c, const T *b0,
             }
             w_m = W, bz_m = bz;
             by_m = by_0, by_0 = by_p, u_m = u_0, u_0 = u_p;
-        }
+        };
+        each_row<CR>(sizeof(T) == 8 ? g.ny - y : CR, row);
         if (i >= 2) cell += g.plane;
     }
     cp_async_wait<0>();
@@ -1038,26 +1062,47 @@ int resident(K k, int threads, size_t bytes) {
 
 bool march3d_supported(int dims, int passes) { return dims == 3 && passes >= 0 && passes <= 1; }
 
-template <typename T, int PASSES, bool HJ>
-void run_source(const Geo &g, const Coef<T> &c, const T *const B[3], const T *const J[3], T *const out[3],
-                cudaStream_t s) {
-    constexpr size_t bytes = (size_t)SOURCE1_RS * (HJ ? 6 : 3) * CPL * sizeof(T);
-    static const int res = resident(k3_source1<T, PASSES, HJ>, CNT, bytes);
-    int zseg;
-    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg, 0.6);
-    k3_source1<T, PASSES, HJ><<<grid, CNT, bytes, s>>>(g, c, B[0], B[1], B[2], HJ ? J[0] : nullptr, HJ ? J[1] : nullptr,
-                                                       HJ ? J[2] : nullptr, out[0], out[1], out[2], zseg);
+// four rows per thread, in the shortest segments, are at most a quarter of the
+// chip's warp schedulers' worth of warps: one row per thread then (128 x 127 x 1 FP64,
+// m = 4: 147 us a step with four)
+bool one_row(const Geo &g) {
+    const double tiles = (double)((g.nx + CX - 1) / CX) * (double)((g.ny + 4 * CW - 1) / (4 * CW));
+    return tiles * CW * g.nz <= sm_count();
 }
 
+template <typename T, int PASSES, bool HJ, int CR>
+void run_source(const Geo &g, const Coef<T> &c, const T *const B[3], const T *const J[3], T *const out[3],
+                cudaStream_t s) {
+    constexpr size_t bytes = (size_t)SOURCE1_RS * (HJ ? 6 : 3) * cpl(CR) * sizeof(T);
+    static const int res = resident(k3_source1<T, PASSES, HJ, CR>, CNT, bytes);
+    int zseg;
+    const dim3 grid = grid_of(g, CX, CR * CW, res, &zseg, 0.6);
+    k3_source1<T, PASSES, HJ, CR><<<grid, CNT, bytes, s>>>(g, c, B[0], B[1], B[2], HJ ? J[0] : nullptr,
+                                                           HJ ? J[1] : nullptr, HJ ? J[2] : nullptr, out[0], out[1],
+                                                           out[2], zseg);
+}
+template <typename T, int PASSES, bool HJ>
+void run_source1(const Geo &g, const Coef<T> &c, const T *const B[3], const T *const J[3], T *const out[3],
+                 cudaStream_t s) {
+    if (one_row(g)) run_source<T, PASSES, HJ, 1>(g, c, B, J, out, s);
+    else run_source<T, PASSES, HJ, 4>(g, c, B, J, out, s);
+}
+
+template <typename T, bool UPD, int CR>
+void run_sweep(const Geo &g, const Coef<T> &c, const T *const dEp[3], const T *const in[3], T *const out[3],
+               cudaStream_t s) {
+    constexpr size_t bytes = (size_t)SWEEP1_RS * 3 * cpl(CR) * sizeof(T);
+    static const int res = resident(k3_sweep1<T, UPD, CR>, CNT, bytes);
+    int zseg;
+    const dim3 grid = grid_of(g, CX, CR * CW, res, &zseg, 0.6);
+    k3_sweep1<T, UPD, CR><<<grid, CNT, bytes, s>>>(g, c, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0], out[1],
+                                                   out[2], zseg);
+}
 template <typename T, bool UPD>
 void run_sweep1(const Geo &g, const Coef<T> &c, const T *const dEp[3], const T *const in[3], T *const out[3],
                 cudaStream_t s) {
-    constexpr size_t bytes = (size_t)SWEEP1_RS * 3 * CPL * sizeof(T);
-    static const int res = resident(k3_sweep1<T, UPD>, CNT, bytes);
-    int zseg;
-    const dim3 grid = grid_of(g, CX, CROWS, res, &zseg, 0.6);
-    k3_sweep1<T, UPD><<<grid, CNT, bytes, s>>>(g, c, dEp[0], dEp[1], dEp[2], in[0], in[1], in[2], out[0], out[1],
-                                               out[2], zseg);
+    if (one_row(g)) run_sweep<T, UPD, 1>(g, c, dEp, in, out, s);
+    else run_sweep<T, UPD, 4>(g, c, dEp, in, out, s);
 }
 
 bool pair_path(const Geo &g, float *) { return g.nx % 2 == 0 && g.pitch % 2 == 0; }
@@ -1131,9 +1176,9 @@ int launch_march3d_source(const Geo &g, const Coef<T> &c, const T *const B[3], c
             return 1;
         }
     }
-    if (!J || !J[0]) run_source<T, 0, false>(g, c, B, J, out, s);
-    else if (passes == 1) run_source<T, 1, true>(g, c, B, J, out, s);
-    else run_source<T, 0, true>(g, c, B, J, out, s);
+    if (!J || !J[0]) run_source1<T, 0, false>(g, c, B, J, out, s);
+    else if (passes == 1) run_source1<T, 1, true>(g, c, B, J, out, s);
+    else run_source1<T, 0, true>(g, c, B, J, out, s);
     return 1;
 }
 
