@@ -448,7 +448,7 @@ struct AdjLauncher {
         return b;
     }
     static void run(const Geo &g, const Coef2 &c, const Adj2dArgs<float> &a, cudaStream_t s) {
-        if (t_adj_rows == 0 && fused2d_tiles(g)) return launch_adj_tile2d<POL, M, P, HJB>(g, c, a, s);
+        if (t_adj_rows == 0 && fused2d_tiles(g, M, P, 8)) return launch_adj_tile2d<POL, M, P, HJB>(g, c, a, s);
         const int width = 2 * NT - 2 * Gm::HC - 2;
         const int strips = (g.nx + width - 1) / width;
         static int sms = -1;

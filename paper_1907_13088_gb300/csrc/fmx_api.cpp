@@ -701,10 +701,11 @@ fmx_status fused_step(fmx_grid *g, int nsteps, StepPre pre = nullptr) {
     // launches go to a second stream, forked from and joined back into the
     // grid's stream (not when profiling: the events time one stream; nor on
     // small grids, whose one launch carries both sets)
+    const int passes = (g->p.filter_target == FMX_FILTER_CURRENT && g->buf.J[0]) ? g->p.filter_passes : 0;
     bool two = false;
     if constexpr (sizeof(T) == 4)
         two = nsteps > 0 && !g->prof && fmx::fused2d_pol_supported(g->geo) && c0.c6 == 1.f / 6.f &&
-              (g->seg_rows > 0 || fmx::fused2d_tiles(g->geo) != 1);
+              (g->seg_rows > 0 || fmx::fused2d_tiles(g->geo, g->p.m, passes) != 1);
     if (pre && nsteps > 0) {
         fmx_status s = pre(g, 0, g->stream);
         if (s != FMX_OK) return s;
@@ -732,7 +733,7 @@ fmx_status fused_step(fmx_grid *g, int nsteps, StepPre pre = nullptr) {
             a.Bo[q] = (T *)g->buf.B[nxt][q];
         }
         a.m = g->p.m;
-        a.passes = (g->p.filter_target == FMX_FILTER_CURRENT && g->buf.J[0]) ? g->p.filter_passes : 0;
+        a.passes = passes;
         cudaEvent_t *ev = g->prof ? profile_events(g, 3) : nullptr;
         int nl;
         if constexpr (sizeof(T) == 4) {

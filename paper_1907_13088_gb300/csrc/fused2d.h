@@ -46,11 +46,12 @@ bool fused2d_pol_supported(const Geo &g);
 // seg_rows: rows per segment (0: one wave of CTAs at the measured occupancy)
 int launch_fused2d_pol(const Geo &g, const Coef<float> &c, const Fused2dArgs<float> &a, cudaStream_t s,
                        cudaEvent_t *ev = nullptr, cudaStream_t s_tm = nullptr, int seg_rows = 0);
+// wide: tiles per SM from which wide grids of few rows go back to the row pipeline.
 // How a grid's FP32 step runs: 0 on the row pipeline, 2 on register tiles
 // (tile2d.cu) with a TE and a TM launch, 1 on register tiles with one launch
 // for both sets (then s_tm is not used).  A launch with seg_rows > 0 or with
 // events takes the path that can honour them; the fields do not depend on it.
-int fused2d_tiles(const Geo &g);
+int fused2d_tiles(const Geo &g, int m, int passes, int wide = 4);
 Fused2dShape fused2d_pol_shape(const Geo &g, int m, int passes, int seg_rows = 0);
 
 // Fused 2D adjoint step (adjoint2d.cu), FP32, TE and TM kernels.  Maps

@@ -85,7 +85,7 @@ struct PolLauncher {
         return sh;
     }
     static void run(const Geo &g, const Coef2 &c, const Fused2dArgs<float> &a, cudaStream_t s) {
-        if (t_rows == 0 && fused2d_tiles(g)) return launch_tile2d<POL, M, P, HJ>(g, c, a, s);
+        if (t_rows == 0 && fused2d_tiles(g, M, P)) return launch_tile2d<POL, M, P, HJ>(g, c, a, s);
         const Fused2dShape sh = shape(g);
         if (g.nx % 2 == 0 && t_l1pf)
             k_pol2d<POL, M, P, HJ, NT, true><<<sh.strips * sh.segments, NT, smem_bytes(), s>>>(a, g, c, sh.width, sh.rows,
@@ -109,7 +109,7 @@ int run_both(const Geo &g, const Coef2 &c, const Fused2dArgs<float> &a, cudaStre
         *sh = PolLauncher<TE, M, P, HJ>::shape(g);
         return 0;
     }
-    if (!t_ev && !t_tm && t_rows == 0 && fused2d_tiles(g) == 1) {
+    if (!t_ev && !t_tm && t_rows == 0 && fused2d_tiles(g, M, P) == 1) {
         launch_tile2d<2, M, P, HJ>(g, c, a, s);
         return 1;
     }

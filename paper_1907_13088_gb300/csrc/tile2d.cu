@@ -12,7 +12,7 @@
 // by one per stage and are the halo.
 //
 // Against the row pipeline (pol_tile.cuh: a barrier per row, 50 rows deep
-// before the first output of a segment is complete) a step has M + 3 barriers
+// before the first output of a segment is complete) a step has M + 2 barriers
 // in all, and neither shared-memory neighbour loads nor ring addresses.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -27,8 +27,9 @@ namespace {
 using namespace tile2d;
 
 // Grids of at most this many cells run both sets in one launch on the grid's
-// own stream: their tiles (48 x 49 columns and rows, both sets) leave SMs free
-// even together, and a step is not worth a second stream's fork and join.
+// own stream: the tiles of both (48 x 49 columns and rows at m = 4, p = 3; 200 at
+// 443^2) are one wave of at most two CTAs per SM, and a step is not worth a second
+// stream's fork and join.
 constexpr double kTileOneLaunchCells = 192.0 * 1024.0;
 
 template <int M, int P, bool HJ>
@@ -296,22 +297,38 @@ FMX_TILE_M(2)
 FMX_TILE_M(3)
 FMX_TILE_M(4)
 
-// Sizes: on the machine's GB300, us per step against the row pipeline (m = 4,
-// p = 3 / vacuum, back to back steps): 64^2 5.4 / 4.3 against 18.5 / 12.3,
-// 512^2 8.8 / 6.6 against 22.6 / 16.4, 1024^2 18.2 / 13.0 against 32.8 / 25.0,
-// 1400^2 37.8 / 25.5 against 47.0 / 34.6, 2048^2 79.3 / 58.4 against 84.2 /
-// 58.6, 4096^2 315 / 233 against 234 / 165.  The tiles recompute 1.75 cells
-// per cell (p = 3), the row pipeline 1.22 on a grid large enough for long
-// segments whose rows it can prefetch from HBM, so the line lies where a
-// step's 60 bytes per cell reach twice the L2.
-int fused2d_tiles(const Geo &g) {
+// Sizes: us per step against the row pipeline (m = 4, p = 3 / vacuum, back to back
+// steps): 64^2 4.7 / 4.0 against 18.5 / 12.3, 512^2 8.8 / 6.6 against 22.6 / 16.4,
+// 1024^2 18.2 / 13.0 against 32.8 / 25.0, 1400^2 37.8 / 25.5 against 47.0 / 34.6,
+// 2048^2 79.3 / 58.4 against 84.2 / 58.6, 4096^2 315 / 233 against 234 / 165.  The
+// tiles recompute 1.75 cells per cell (p = 3), the row pipeline 1.22 on a grid
+// large enough for long segments whose rows it can prefetch from HBM, so the line
+// lies where a step's 60 bytes per cell (48 without a current, where the two meet
+// a little earlier) reach twice the L2.
+// Wide grids of few rows: a tile holds 64 rows of warps however few it needs, and
+// with several waves of such tiles the row pipeline is ahead while one segment of
+// it takes the whole height (about its 3m + 2p + 8 warm-up rows).  Tiles against
+// rows, n_x = 50000, m = 4, p = 3: 8 rows 26.4 / 21.8, 24 rows 34.0 / 29.9, 28 rows
+// 37.0 / 40.7; vacuum 20 rows 22.6 / 20.5, 28 rows 26.8 / 25.8; m = 1, p = 0: 8 rows
+// 14.5 / 9.0, 20 rows 15.9 / 14.5, 24 rows 16.4 / 18.2; n_x = 400000, m = 4, p = 3, 8 rows
+// 242 / 121; n_x = 20001, 8 rows 13.7 / 21.8.  So from `wide` tiles per SM on; 4, and
+// 8 for the adjoint (us per step of both sets and jbar, m = 4, p = 3, 8 rows: n_x =
+// 50000 78.7 / 84.4, 100000 96.8 / 92.7, 400000 252 / 208).
+int fused2d_tiles(const Geo &g, int m, int passes, int wide) {
     static const long long l2 = [] {
         int dev = 0, v = 0;
         cudaGetDevice(&dev);
         return cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev) == cudaSuccess && v > 0 ? (long long)v : 1LL << 27;
     }();
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0 ? v : 1;
+    }();
     const double cells = (double)g.nx * (double)g.ny;
     if (60.0 * cells > 2.0 * (double)l2) return 0;
+    const int warm = 3 * m + 2 * passes + 8;
+    if (g.nx >= 48LL * wide * sms && g.ny <= (warm > 20 ? warm : 20)) return 0;
     return cells <= kTileOneLaunchCells ? 1 : 2;
 }
 
