@@ -219,7 +219,7 @@ fmx_status fmx_step(fmx_grid *g, int nsteps);
 /* Applies `passes` binomial passes along every active axis to the
  * components in mask (FMX_E, FMX_B, FMX_J bits), in place on the current
  * state -- the "post-process the fields and currents" option of Sec. 5.
- * Enqueued on the stream.  Errors: FMX_ESTATE, FMX_EINVAL. */
+ * Writes those components and workspace only.  Enqueued on the stream.  Errors: FMX_ESTATE, FMX_EINVAL. */
 fmx_status fmx_filter(fmx_grid *g, unsigned mask, int passes);
 
 /* Copies the components in mask (FMX_E/FMX_B/FMX_J bits; dst indexed
@@ -540,10 +540,12 @@ fmx_status fmx_step_static(const fmx_params *p, void *const *E, void *const *B, 
  *     2D fused engine (the TE and TM kernels of the step and of the adjoint
  *     step) each march over, a grid of at most that many rows taking one
  *     segment; every segment recomputes a few warm-up rows of the row
- *     pipeline.  0 (default): a grid whose 60 bytes per cell are at most
- *     twice the L2 runs on register tiles instead of row segments; elsewhere as many segments as fill one wave of CTAs at the
- *     kernels' occupancy, but none shorter than 3m + 2p + 8 rows (p: the
- *     current's filter passes, 0 without a current).  Same results to the
+ *     pipeline.  0 (default): a grid whose 60 bytes per
+ *     cell are at most twice the L2 runs on register tiles instead of row
+ *     segments, unless it is wide and of few rows; elsewhere as many segments
+ *     as fill one wave of CTAs at the kernels' occupancy, but none shorter
+ *     than 3m + 2p + 8 rows (p: the current's filter passes, 0 without a
+ *     current).  Same results to the
  *     bit.
  * fmx_set_option returns FMX_EINVAL for an unknown or read-only option or a
  * bad value; fmx_get_option returns the value, or -1 (unknown option or NULL

@@ -509,14 +509,11 @@ fmx_status staged_step(fmx_grid *g) {
                     continue;
                 }
             }
-            // the z-marching FP32 sweep can apply E^{n+1} = E^n + dE in its last pass
+            // the z-marching sweep applies E^{n+1} = E^n + dE in its last pass
             if (march && it == g->p.m - 1) {
-                const int n = fmx::launch_march3d_sweep<T>(g->geo, c, dp, in, P.E, g->stream, true);
-                g->launches += n;
-                if (n) {
-                    updated = true;
-                    break;
-                }
+                g->launches += fmx::launch_march3d_sweep<T>(g->geo, c, dp, in, P.E, g->stream, true);
+                updated = true;
+                break;
             }
             T *out[3];
             for (int q = 0; q < 3; ++q) out[q] = in[0] == P.dEa[0] ? P.dEb[q] : P.dEa[q];
@@ -573,8 +570,8 @@ fmx_status staged_step(fmx_grid *g) {
     }
     {
         const T *e[3] = {P.E[0], P.E[1], P.E[2]};
-        const int n = march ? fmx::launch_march3d_faraday<T>(g->geo, c, e, P.B, g->stream) : 0;
-        g->launches += n ? n : fmx::launch_faraday<T>(g->geo, g->p.dims, c, P.E, P.B, g->stream);
+        g->launches += march ? fmx::launch_march3d_faraday<T>(g->geo, c, e, P.B, g->stream)
+                             : fmx::launch_faraday<T>(g->geo, g->p.dims, c, P.E, P.B, g->stream);
     }
     s = check_launch(g, "staged step launch");
     if (s != FMX_OK) return s;

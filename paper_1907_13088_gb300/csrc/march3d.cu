@@ -1162,7 +1162,7 @@ int launch_march3d_sweeps2(const Geo &g, const Coef<T> &c, const T *const dEp[3]
             return 1;
         }
     }
-    return 0;  // FP64, odd n_x or a small grid: the caller runs the sweeps one per pass
+    return 0;  // FP64 or odd n_x: the caller runs the sweeps one per pass
 }
 
 template <typename T>
@@ -1189,7 +1189,7 @@ int launch_march3d_faraday(const Geo &g, const Coef<T> &c, const T *const E[3], 
             constexpr size_t bytes = (size_t)FAR_RS * 3 * PL2 * sizeof(float);
             static const int res = resident(k3_faraday2, NTH, bytes);
             int zseg;
-    const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
+            const dim3 grid = grid_of(g, TX2, TY, res, &zseg);
             k3_faraday2<<<grid, dim3(TXP, TY), bytes, s>>>(g, coef3p(c), E[0], E[1], E[2], B[0], B[1], B[2], zseg);
             return 1;
         }

@@ -249,7 +249,7 @@ __device__ __forceinline__ void pol_tile(const Fused2dArgs<float> &a, const Geo 
         if (POL == TM) pf1[k] = ld2(inB1, of);
         adv(of);
     };
-    // rows r0 .. r0 + depth - 1 of each stream (r0 is a multiple of 4)
+    // rows r0 .. r0 + depth - 1 of each stream (buffers go by r - r0)
 #pragma unroll
     for (int k = 0; k < PJ; ++k) ldJ(k);
 #pragma unroll
@@ -273,7 +273,9 @@ __device__ __forceinline__ void pol_tile(const Fused2dArgs<float> &a, const Geo 
 #pragma unroll
         for (int k = 0; k < PE; ++k) pe1[k] = z2;
     }
-    int b0 = ALIGN ? ((r0 % D0) + D0) % D0 : 0;  // dE' ring slot of row r0 (a multiple of 4)
+    // dE' ring slot of row r0.  Slots and unroll go by r - r0: b0 has to be a multiple
+    // of 4 (r0 need not; without ALIGN b0 is 0), and r1 - r0 is one
+    int b0 = ALIGN ? ((r0 % D0) + D0) % D0 : 0;
     // With D0 = 12 the dE' ring is addressed through the bases of its three
     // 4-row groups, rotated once per block of four rows, so that every slot a
     // row touches is a compile-time offset from one of them (no per-access
