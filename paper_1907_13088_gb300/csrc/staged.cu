@@ -89,10 +89,13 @@ __device__ __forceinline__ T filter_taps(const T *v) {
 // written by its own CTA only, once all of them are loaded).  So the filter takes
 // the workspace's one spare component array and none of the caller's others.  A
 // grid of one tile is its own halo: one launch, ring = nullptr.
-// FP32 is bound by memory: each cell is read and written once, and the halos (P =
-// 1: 6%).  FP64 is bound by its 2 (2P + 1) operations per cell, which is why the x
-// taps are evaluated once per row of the tile (9% more rows than cells at P = 3)
-// and small grids are cut into smaller tiles, over more SMs.
+// Each cell is read and written once, and the halos (P = 1: 6%).  FP32 is bound by
+// issue (72%): 1536 x 1200, E and B, P = 1: 12 + 22 us launched cold, 27 warm (two passes
+// through a second array 35 + 33, one launch per component, axis and pass 12 x 10).
+// FP64 is bound by its 2 (2P + 1) operations per cell, which is why the x taps are
+// evaluated once per row of the tile (9% more rows than cells at P = 3) and small
+// grids are cut into smaller tiles, over more SMs (same grid, P = 2: 258 us with the
+// x taps of a row evaluated by each group of rows, 239 now).
 // ring_size is how much of it a tile of a component takes, ring_cell the cell of
 // its element e: P rows below and above with their corners, then P columns left
 // and right.

@@ -298,9 +298,9 @@ FMX_TILE_M(3)
 FMX_TILE_M(4)
 
 // Sizes: us per step against the row pipeline (m = 4, p = 3 / vacuum, back to back
-// steps): 64^2 4.7 / 4.0 against 18.5 / 12.3, 512^2 8.8 / 6.6 against 22.6 / 16.4,
-// 1024^2 18.2 / 13.0 against 32.8 / 25.0, 1400^2 37.8 / 25.5 against 47.0 / 34.6,
-// 2048^2 79.3 / 58.4 against 84.2 / 58.6, 4096^2 315 / 233 against 234 / 165.  The
+// steps): 64^2 5.2 / 4.2 against 16.8 / 12.4, 512^2 8.8 / 6.7 against 22.9 / 18.5,
+// 1024^2 18.2 / 13.0 against 30.8 / 22.6, 1400^2 37.8 / 25.7 against 47.2 / 32.6,
+// 2048^2 78.6 / 58.3 against 82.2 / 59.1, 4096^2 315 / 233 against 234 / 165.  The
 // tiles recompute 1.75 cells per cell (p = 3), the row pipeline 1.22 on a grid
 // large enough for long segments whose rows it can prefetch from HBM, so the line
 // lies where a step's 60 bytes per cell (48 without a current, where the two meet
