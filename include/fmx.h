@@ -540,13 +540,11 @@ fmx_status fmx_step_static(const fmx_params *p, void *const *E, void *const *B, 
  *     2D fused engine (the TE and TM kernels of the step and of the adjoint
  *     step) each march over, a grid of at most that many rows taking one
  *     segment; every segment recomputes a few warm-up rows of the row
- *     pipeline.  0 (default): a grid whose 60 bytes per
- *     cell are at most twice the L2 runs on register tiles instead of row
- *     segments, unless it is wide and of few rows; elsewhere as many segments
- *     as fill one wave of CTAs at the kernels' occupancy, but none shorter
- *     than 3m + 2p + 8 rows (p: the current's filter passes, 0 without a
- *     current).  Same results to the
- *     bit.
+ *     pipeline.  0 (default): a grid whose 60 bytes per cell are at most twice
+ *     the L2 runs on register tiles instead of row segments, unless it is wide
+ *     and of few rows; elsewhere as many segments as fill one wave of CTAs at
+ *     the kernels' occupancy, but none shorter than 3m + 2p + 8 rows (p: the
+ *     current's filter passes, 0 without a current).  Same results to the bit.
  * fmx_set_option returns FMX_EINVAL for an unknown or read-only option or a
  * bad value; fmx_get_option returns the value, or -1 (unknown option or NULL
  * grid). */
